@@ -3,20 +3,17 @@
 // the Slotboom-transformed Nernst-Planck equations (Sec 2.1, 7-point
 // harmonic-mean stencil of Sec 3.1).
 //
-// Operators are matrix-free: per grid level, face coefficients cx[p] (face to
-// the +x neighbour, wrapping; zero across a no-flux wall), cy[p], cz[p] (face
-// to +z; on the top plane the face to the upper Dirichlet plane) and czlo[p]
-// (face to the lower Dirichlet plane, plane 0 only);
-//   (A u)_p = sum_faces c (u_p - u_nbr),  Dirichlet neighbours moved to b.
+// Operators are matrix-free (mg_pcg.cuh: level layout, kernels).
 // Multigrid (replacing the paper's external algebraic multigrid, Sec 3.3):
-// cells are aggregated 2x2x2 (per axis while even and >= 4); the coarse
-// operator is the Galerkin product with piecewise-constant interpolation,
-// i.e. coarse face coefficients are sums of the fine faces between two
-// aggregates; restriction sums the 8 fine residuals, prolongation adds the
-// coarse value.  One V(1,1) cycle with red-black sweeps (red-black before,
-// black-red after, so the cycle is a symmetric operator) preconditions CG;
-// the coarsest level gets 40 symmetric sweeps in one CTA.  All dot products
-// use a fixed-shape two-stage reduction, so results are bitwise reproducible.
+// cells are aggregated 2x2x2 (per axis while even and >= 4, else 3 or 5); the
+// coarse operator is the Galerkin product with piecewise-constant
+// interpolation, i.e. coarse face coefficients are sums of the fine faces
+// between two aggregates; restriction sums the fine residuals, prolongation
+// adds the coarse value.  One V(2,2) cycle with red-black sweeps (red, black,
+// red, black before, black, red, black, red after, so the cycle is a
+// symmetric operator) preconditions CG; the coarsest level gets 40 symmetric
+// sweeps.  All dot products use a fixed-shape two-stage reduction, so results
+// are bitwise reproducible.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -26,27 +23,6 @@
 #include "pnp_internal.h"
 
 namespace pnp {
-
-struct Op {
-    int nx, ny, nz;
-    const double *cx, *cy, *cz, *czlo;
-    const double *dg = nullptr;    // optional extra diagonal (Poisson-Boltzmann screening)
-};
-
-struct Level {
-    int nx, ny, nz;
-    size_t n;
-    int fx, fy, fz;                // aggregation factors to the next level
-    double *cx, *cy, *cz, *czlo;   // operator being solved (Poisson or NP)
-    double *pcx, *pcy, *pcz, *pczlo;   // Poisson copy (built once)
-    double *dg;                    // diagonal term of the screened Poisson operator
-    double *x, *b, *r;
-};
-
-constexpr int kRedBlocks = 512;
-constexpr int kCoarseSweeps = 40;
-constexpr double kCoarseScale = 1.8;
-constexpr double kMixStepLimit = 0.2;     // |step in ln rho| of PNP_MIX_GEOMETRIC_LIMITED
 
 // device-side record of a solve (written by the loop-control kernels)
 struct DevStats {
@@ -80,9 +56,18 @@ struct AaCtl {
 };
 constexpr int kAaBacktrack = 8;    // step halvings after the restart from the plain iterate
 
+}  // namespace pnp
+
+#include "mg_pcg.cuh"
+
+namespace pnp {
+
 struct GummelState {
     std::vector<Level> lv;
-    double *mu = nullptr, *rho_new = nullptr;
+    int lt = 0;                    // first level of the one-CTA tail (or the coarsest, without one)
+    bool tail = false;
+    size_t tail_smem = 0;
+    double *mu = nullptr;
     double *phi = nullptr, *rho = nullptr;    // solve state the graph works on
     DevStats *stats = nullptr;
     int *keep_q = nullptr;                    // valences and fixed charge used by the graph
@@ -91,7 +76,9 @@ struct GummelState {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     double *rhs = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *pv = nullptr, *Ap = nullptr;
-    double *partial = nullptr;     // kRedBlocks
+    double *z2 = nullptr;          // second buffer of z on odd grids (z otherwise)
+    double *em = nullptr;          // exp(-(q phi + mu)) of the current species
+    double *partial = nullptr;     // four sets of kDotBlocks partial sums
     double *lam = nullptr, *prev = nullptr;   // PNP_MIX_ADAPTIVE: per-point factor and last step
     double *scal = nullptr;        // device scalars
     // Anderson mixing (depth m > 0): history of m + 1 iterates x = (phi, ln rho)
@@ -103,189 +90,16 @@ struct GummelState {
     double *phase = nullptr;          // PNP_FLAG_PHASE_TIMING: ns per phase, then the last mark
     unsigned long long *dmax = nullptr;
     size_t bytes = 0;
-    bool poisson_ready = false;
     bool shift = false;            // operators carry the levels' dg while capturing
 };
 
-enum { S_RZ = 0, S_PAP, S_RR, S_ALPHA, S_BETA, S_RZNEW, S_BB, S_TGT, S_COUNT };
-
-__device__ __forceinline__ size_t pidx(int i, int j, int k, int nx, int ny) {
-    return ((size_t)k * ny + j) * nx + i;
-}
-
-__device__ __forceinline__ double op_diag(const Op &A, int i, int j, int k, size_t p) {
-    const int im = i == 0 ? A.nx - 1 : i - 1, jm = j == 0 ? A.ny - 1 : j - 1;
-    double d = A.cx[p] + A.cy[p] + A.cz[p];
-    d += A.cx[pidx(im, j, k, A.nx, A.ny)] + A.cy[pidx(i, jm, k, A.nx, A.ny)];
-    d += k > 0 ? A.cz[p - (size_t)A.nx * A.ny] : A.czlo[p];
-    if (A.dg) d += A.dg[p];
-    return d;
-}
-
-__device__ __forceinline__ double op_nbr(const Op &A, const double *__restrict__ u, int i, int j, int k, size_t p) {
-    const int ip = i + 1 == A.nx ? 0 : i + 1, im = i == 0 ? A.nx - 1 : i - 1;
-    const int jp = j + 1 == A.ny ? 0 : j + 1, jm = j == 0 ? A.ny - 1 : j - 1;
-    const size_t plane = (size_t)A.nx * A.ny;
-    const size_t pxm = pidx(im, j, k, A.nx, A.ny), pym = pidx(i, jm, k, A.nx, A.ny);
-    double s = A.cx[p] * u[pidx(ip, j, k, A.nx, A.ny)] + A.cx[pxm] * u[pxm];
-    s += A.cy[p] * u[pidx(i, jp, k, A.nx, A.ny)] + A.cy[pym] * u[pym];
-    if (k + 1 < A.nz) s += A.cz[p] * u[p + plane];
-    if (k > 0) s += A.cz[p - plane] * u[p - plane];
-    return s;
-}
+constexpr int kRedBlocks = 512;
+constexpr double kMixStepLimit = 0.2;     // |step in ln rho| of PNP_MIX_GEOMETRIC_LIMITED
 
 #define GRID_LOOP(p, n) for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < (n); p += (size_t)gridDim.x * blockDim.x)
 
-__global__ void k_residual(Op A, const double *__restrict__ x, const double *__restrict__ b, double *__restrict__ r) {
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-        r[p] = b[p] - (op_diag(A, i, j, k, p) * x[p] - op_nbr(A, x, i, j, k, p));
-    }
-}
-
-__global__ void k_apply(Op A, const double *__restrict__ x, double *__restrict__ y) {
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-        y[p] = op_diag(A, i, j, k, p) * x[p] - op_nbr(A, x, i, j, k, p);
-    }
-}
-
-// one colour of a red-black sweep: x_p = (b_p + sum c x_nbr) / diag_p for
-// points with (i + j + k) % 2 == color.  With zero_init the other colour is
-// taken as zero (first sweep from x = 0).
-__global__ void k_color_sweep(Op A, double *__restrict__ x, const double *__restrict__ b, int color) {
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-        if (((i + j + k) & 1) != color) continue;
-        x[p] = (b[p] + op_nbr(A, x, i, j, k, p)) / op_diag(A, i, j, k, p);
-    }
-}
-
-// coarsest level: x = 0, then kCoarseSweeps symmetric (red, black, black, red) sweeps in one CTA
-__global__ void k_coarse_solve(Op A, double *__restrict__ x, const double *__restrict__ b) {
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    for (size_t p = threadIdx.x; p < n; p += blockDim.x) x[p] = 0.0;
-    __syncthreads();
-    for (int s = 0; s < kCoarseSweeps; ++s) {
-        const int order[4] = {0, 1, 1, 0};
-        for (int c = 0; c < 4; ++c) {
-            for (size_t p = threadIdx.x; p < n; p += blockDim.x) {
-                const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-                if (((i + j + k) & 1) != order[c]) continue;
-                x[p] = (b[p] + op_nbr(A, x, i, j, k, p)) / op_diag(A, i, j, k, p);
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// coarse face coefficients: sums of the fine faces leaving each aggregate
-__global__ void k_coarsen(Op F, int fx, int fy, int fz, int cnx, int cny, int cnz, double *__restrict__ cx,
-                          double *__restrict__ cy, double *__restrict__ cz, double *__restrict__ czlo) {
-    const size_t n = (size_t)cnx * cny * cnz;
-    GRID_LOOP(q, n) {
-        const int I = q % cnx, J = (q / cnx) % cny, K = q / ((size_t)cnx * cny);
-        double sx = 0, sy = 0, sz = 0, sl = 0;
-        for (int c = 0; c < fz; ++c)
-            for (int b = 0; b < fy; ++b)
-                for (int a = 0; a < fx; ++a) {
-                    const int i = I * fx + a, j = J * fy + b, k = K * fz + c;
-                    const size_t p = pidx(i, j, k, F.nx, F.ny);
-                    if (a == fx - 1) sx += F.cx[p];
-                    if (b == fy - 1) sy += F.cy[p];
-                    if (c == fz - 1) sz += F.cz[p];
-                    if (c == 0 && K == 0) sl += F.czlo[p];
-                }
-        cx[q] = sx;
-        cy[q] = sy;
-        cz[q] = sz;
-        czlo[q] = sl;
-    }
-}
-
-__global__ void k_restrict(const double *__restrict__ rf, int nx, int ny, int fx, int fy, int fz, int cnx, int cny,
-                           int cnz, double *__restrict__ bc) {
-    const size_t n = (size_t)cnx * cny * cnz;
-    GRID_LOOP(q, n) {
-        const int I = q % cnx, J = (q / cnx) % cny, K = q / ((size_t)cnx * cny);
-        double s = 0;
-        for (int c = 0; c < fz; ++c)
-            for (int b = 0; b < fy; ++b)
-                for (int a = 0; a < fx; ++a) s += rf[pidx(I * fx + a, J * fy + b, K * fz + c, nx, ny)];
-        bc[q] = s;
-    }
-}
-
-// x_fine += scale * x_coarse (piecewise constant); scale > 1 compensates the
-// weak correction of piecewise-constant interpolation
-__global__ void k_prolong_add(double *__restrict__ xf, int nx, int ny, int nz, int fx, int fy, int fz, int cnx,
-                              int cny, const double *__restrict__ xc, double scale) {
-    const size_t n = (size_t)nx * ny * nz;
-    GRID_LOOP(p, n) {
-        const int i = p % nx, j = (p / nx) % ny, k = p / ((size_t)nx * ny);
-        xf[p] += scale * xc[pidx(i / fx, j / fy, k / fz, cnx, cny)];
-    }
-}
-
 __global__ void k_fill(double *__restrict__ a, double v, size_t n) {
     GRID_LOOP(p, n) a[p] = v;
-}
-
-// deterministic dot product, stage 1: fixed grid of kRedBlocks blocks
-__global__ void k_dot_partial(const double *__restrict__ a, const double *__restrict__ b, size_t n,
-                              double *__restrict__ partial) {
-    __shared__ double sh[256];
-    double s = 0;
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x)
-        s += a[p] * b[p];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-// stage 2: one block sums the partials into scal[slot]
-__global__ void k_dot_final(const double *__restrict__ partial, double *__restrict__ scal, int slot) {
-    __shared__ double sh[kRedBlocks];
-    for (int t = threadIdx.x; t < kRedBlocks; t += blockDim.x) sh[t] = partial[t];
-    __syncthreads();
-    for (int w = kRedBlocks / 2; w > 0; w >>= 1) {
-        for (int t = threadIdx.x; t < w; t += blockDim.x) sh[t] += sh[t + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) scal[slot] = sh[0];
-}
-
-__global__ void k_scalars_alpha(double *scal) {
-    scal[S_ALPHA] = scal[S_RZ] / scal[S_PAP];
-}
-
-__global__ void k_scalars_beta(double *scal) {
-    scal[S_BETA] = scal[S_RZNEW] / scal[S_RZ];
-    scal[S_RZ] = scal[S_RZNEW];
-}
-
-// x += alpha p ; r -= alpha Ap
-__global__ void k_update_xr(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                            const double *__restrict__ Ap, const double *__restrict__ scal, size_t n) {
-    const double a = scal[S_ALPHA];
-    GRID_LOOP(k, n) {
-        x[k] += a * p[k];
-        r[k] -= a * Ap[k];
-    }
-}
-
-// p = z + beta p
-__global__ void k_update_p(double *__restrict__ p, const double *__restrict__ z, const double *__restrict__ scal,
-                           size_t n) {
-    const double b = scal[S_BETA];
-    GRID_LOOP(k, n) p[k] = z[k] + b * p[k];
 }
 
 __global__ void k_copy(double *__restrict__ d, const double *__restrict__ s, size_t n) {
@@ -308,7 +122,7 @@ __global__ void k_poisson_coefs(PhysConst c, double *cx, double *cy, double *cz,
         cx[p] = (c.bcx == PNP_BC_NOFLUX && i == c.nx - 1) ? 0.0 : 1.0;
         cy[p] = (c.bcy == PNP_BC_NOFLUX && j == c.ny - 1) ? 0.0 : 1.0;
         cz[p] = 1.0;
-        czlo[p] = k == 0 ? 1.0 : 0.0;
+        if (k == 0) czlo[p] = 1.0;
     }
 }
 
@@ -334,9 +148,8 @@ __global__ void k_scr_rhs(Op A, PhysConst c, const double *__restrict__ rho, int
                           const double *__restrict__ rho_f, const double *__restrict__ phi, double *__restrict__ rhs,
                           double *__restrict__ dg) {
     const size_t n = (size_t)c.nx * c.ny * c.nz;
-    const size_t plane = (size_t)c.nx * c.ny;
     GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / plane;
+        const Pt t = pt_flat(A, (unsigned)p);
         double ch = rho_f ? rho_f[p] : 0.0, sc = 0.0;
         for (int a = 0; a < s; ++a) {
             const double r = rho[a * n + p];
@@ -344,9 +157,9 @@ __global__ void k_scr_rhs(Op A, PhysConst c, const double *__restrict__ rho, int
             sc += (double)(q[a] * q[a]) * r;
         }
         double b = 4.0 * M_PI * c.lB * ch;
-        if (k == 0) b += c.phi_lo;
-        if (k + 1 == c.nz) b += c.phi_hi;
-        rhs[p] = b - (op_diag(A, i, j, k, p) * phi[p] - op_nbr(A, phi, i, j, k, p));
+        if (t.k == 0) b += c.phi_lo;
+        if (t.k + 1 == c.nz) b += c.phi_hi;
+        rhs[p] = b - (__dmul_rn(op_diag(A, t), phi[p]) - op_nbr(A, phi, phi, t));
         dg[p] = 4.0 * M_PI * c.lB * sc;
     }
 }
@@ -382,65 +195,61 @@ struct NpConst {
     double D, q, Dlo, Dhi, rlo, rhi;
 };
 
-// Slotboom coefficients (Sec 2.1) and the harmonic-mean face coefficients
-// (Sec 3.1): Dbar = D exp(-(q phi + mu)); faces to the Dirichlet planes use
-// the reservoir value D exp(-(q phi_face + mu_b)).  Also writes the Dirichlet
-// right-hand side and the initial guess rhobar = rho exp(q phi + mu).
-__global__ void k_np_setup(PhysConst c, NpConst s, const double *__restrict__ phi, const double *__restrict__ mu,
-                           const double *__restrict__ rho, double *__restrict__ cx, double *__restrict__ cy,
-                           double *__restrict__ cz, double *__restrict__ czlo, double *__restrict__ b,
-                           double *__restrict__ x0, int *__restrict__ flag) {
-    const size_t n = (size_t)c.nx * c.ny * c.nz;
-    const size_t plane = (size_t)c.nx * c.ny;
+// exp(-(q phi + mu)) of the Slotboom mobility Dbar = D exp(-(q phi + mu)) (Sec
+// 2.1) and the initial guess rhobar = rho exp(q phi + mu).  An FP64 exponential
+// costs some 25 multiply-adds and GB300 issues two a clock and SM, so it is
+// taken once per point and kept: the faces (k_np_faces) and the way back
+// (k_np_finish) read it (one exponential per point and sign instead of six).
+__global__ void k_np_mobility(size_t n, NpConst s, const double *__restrict__ phi, const double *__restrict__ mu,
+                              const double *__restrict__ rho, double *__restrict__ em, double *__restrict__ x0,
+                              int *__restrict__ flag) {
     bool bad = false;
     GRID_LOOP(p, n) {
-        const int i = p % c.nx, j = (p / c.nx) % c.ny, k = p / plane;
-        auto Db = [&](size_t t) { return s.D * exp(-(s.q * phi[t] + mu[t])); };
-        const double d0 = Db(p);
-        const size_t pxp = pidx(i + 1 == c.nx ? 0 : i + 1, j, k, c.nx, c.ny);
-        const size_t pyp = pidx(i, j + 1 == c.ny ? 0 : j + 1, k, c.nx, c.ny);
-        double vx = 0, vy = 0;
-        if (!(c.bcx == PNP_BC_NOFLUX && i == c.nx - 1)) {
-            const double d1 = Db(pxp);
-            vx = 2.0 * d0 * d1 / (d0 + d1);
-        }
-        if (!(c.bcy == PNP_BC_NOFLUX && j == c.ny - 1)) {
-            const double d1 = Db(pyp);
-            vy = 2.0 * d0 * d1 / (d0 + d1);
-        }
-        double vz;
-        if (k + 1 < c.nz) {
-            const double d1 = Db(p + plane);
-            vz = 2.0 * d0 * d1 / (d0 + d1);
-        } else {
-            vz = 2.0 * d0 * s.Dhi / (d0 + s.Dhi);
-        }
-        const double vl = k == 0 ? 2.0 * d0 * s.Dlo / (d0 + s.Dlo) : 0.0;
-        cx[p] = vx;
-        cy[p] = vy;
-        cz[p] = vz;
-        czlo[p] = vl;
-        double bv = 0;
-        if (k == 0) bv += vl * s.rlo;
-        if (k + 1 == c.nz) bv += vz * s.rhi;
-        b[p] = bv;
-        const double x = rho[p] * exp(s.q * phi[p] + mu[p]);
+        const double e = s.q * phi[p] + mu[p];
+        const double m = exp(-e), d = s.D * m;
+        const double x = rho[p] * exp(e);
+        em[p] = m;
         x0[p] = x;
-        if (!isfinite(d0) || !isfinite(x) || !(d0 > 0)) bad = true;
+        if (!isfinite(d) || !isfinite(x) || !(d > 0)) bad = true;
     }
     if (bad) atomicOr(flag, kFlagOverflow);
 }
 
-// rho* = rhobar exp(-(q phi + mu)); relaxation (linear or geometric); track
-// max |rho_new - rho| / rho_b
-__global__ void k_np_finish(size_t n, double q, double l2, int mix, double inv_rb, const double *__restrict__ phi,
-                            const double *__restrict__ mu, const double *__restrict__ rbar, double *__restrict__ rho,
-                            double *__restrict__ lam, double *__restrict__ prev,
+// Harmonic-mean face coefficients (Sec 3.1) of the mobilities D em; faces to the
+// Dirichlet planes use the reservoir value D exp(-(q phi_face + mu_b)).  Also
+// writes the Dirichlet right-hand side.
+__global__ void k_np_faces(PhysConst c, NpConst s, Op A, const double *__restrict__ em, double *__restrict__ cx,
+                           double *__restrict__ cy, double *__restrict__ cz, double *__restrict__ czlo,
+                           double *__restrict__ b) {
+    const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= A.n) return;
+    const Pt q = pt_flat(A, p);
+    const double d0 = s.D * em[p];
+    auto mean = [&](double d1) { return 2.0 * d0 * d1 / (d0 + d1); };
+    cx[p] = c.bcx == PNP_BC_NOFLUX && q.i == c.nx - 1 ? 0.0 : mean(s.D * em[nbr_xp(A, q)]);
+    cy[p] = c.bcy == PNP_BC_NOFLUX && q.j == c.ny - 1 ? 0.0 : mean(s.D * em[nbr_yp(A, q)]);
+    const double vz = mean(q.k + 1 < c.nz ? s.D * em[p + A.plane] : s.Dhi);
+    cz[p] = vz;
+    double bv = 0;
+    if (q.k == 0) {
+        const double vl = mean(s.Dlo);
+        czlo[p] = vl;
+        bv += vl * s.rlo;
+    }
+    if (q.k + 1 == c.nz) bv += vz * s.rhi;
+    b[p] = bv;
+}
+
+// rho* = rhobar exp(-(q phi + mu)) (the exponential kept in em); relaxation
+// (linear or geometric); track max |rho_new - rho| / rho_b
+__global__ void k_np_finish(size_t n, double l2, int mix, double inv_rb, const double *__restrict__ em,
+                            const double *__restrict__ rbar, double *__restrict__ rho, double *__restrict__ lam,
+                            double *__restrict__ prev,
                             unsigned long long *__restrict__ dmax, int *__restrict__ flag) {
     double m = 0;
     bool bad = false;
     GRID_LOOP(p, n) {
-        const double rs = rbar[p] * exp(-(q * phi[p] + mu[p]));
+        const double rs = rbar[p] * em[p];
         const double old = rho[p];
         double v;
         if (mix == PNP_MIX_LINEAR) {
@@ -477,114 +286,7 @@ __global__ void k_init_phi(PhysConst c, double *__restrict__ phi) {
 }
 
 
-// first red sweep from x = 0: red points b/diag, black points 0 (replaces a
-// fill and a sweep)
-__global__ void k_sweep_zero(Op A, double *__restrict__ x, const double *__restrict__ b) {
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-        x[p] = ((i + j + k) & 1) ? 0.0 : b[p] / op_diag(A, i, j, k, p);
-    }
-}
-
-// coarse right-hand side = sum of the fine residuals b - A x over each aggregate
-__global__ void k_residual_restrict(Op F, const double *__restrict__ x, const double *__restrict__ b, int fx, int fy,
-                                    int fz, int cnx, int cny, int cnz, double *__restrict__ bc) {
-    const size_t n = (size_t)cnx * cny * cnz;
-    GRID_LOOP(q, n) {
-        const int I = q % cnx, J = (q / cnx) % cny, K = q / ((size_t)cnx * cny);
-        double s = 0;
-        for (int c = 0; c < fz; ++c)
-            for (int bb = 0; bb < fy; ++bb)
-                for (int a = 0; a < fx; ++a) {
-                    const int i = I * fx + a, j = J * fy + bb, k = K * fz + c;
-                    const size_t p = pidx(i, j, k, F.nx, F.ny);
-                    s += b[p] - (op_diag(F, i, j, k, p) * x[p] - op_nbr(F, x, i, j, k, p));
-                }
-        bc[q] = s;
-    }
-}
-
-// coarsest level in shared memory: x = 0, then kCoarseSweeps symmetric
-// red-black sweeps; n <= kCoarseMax
-constexpr int kCoarseMax = 1024;
-__global__ void k_coarse_smem(Op A, double *__restrict__ x_out, const double *__restrict__ b_in) {
-    extern __shared__ double csm[];
-    const int n = A.nx * A.ny * A.nz;
-    double *x = csm, *b = csm + n, *dg = csm + 2 * n, *cx = csm + 3 * n, *cy = csm + 4 * n, *cz = csm + 5 * n,
-           *cl = csm + 6 * n;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        x[p] = 0.0;
-        b[p] = b_in[p];
-        cx[p] = A.cx[p];
-        cy[p] = A.cy[p];
-        cz[p] = A.cz[p];
-        cl[p] = A.czlo[p];
-    }
-    __syncthreads();
-    const Op S{A.nx, A.ny, A.nz, cx, cy, cz, cl};
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / (A.nx * A.ny);
-        dg[p] = op_diag(S, i, j, k, p) + (A.dg ? A.dg[p] : 0.0);
-    }
-    __syncthreads();
-    const int order[4] = {0, 1, 1, 0};
-    for (int s = 0; s < kCoarseSweeps; ++s)
-        for (int c = 0; c < 4; ++c) {
-            for (int p = threadIdx.x; p < n; p += blockDim.x) {
-                const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / (A.nx * A.ny);
-                if (((i + j + k) & 1) != order[c]) continue;
-                x[p] = (b[p] + op_nbr(S, x, i, j, k, p)) / dg[p];
-            }
-            __syncthreads();
-        }
-    for (int p = threadIdx.x; p < n; p += blockDim.x) x_out[p] = x[p];
-}
-
-// y = A x and the block partial sums of x . y
-__global__ void k_apply_dot(Op A, const double *__restrict__ x, double *__restrict__ y, double *__restrict__ partial) {
-    __shared__ double sh[256];
-    const size_t n = (size_t)A.nx * A.ny * A.nz;
-    double acc = 0;
-    GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / ((size_t)A.nx * A.ny);
-        const double v = op_diag(A, i, j, k, p) * x[p] - op_nbr(A, x, i, j, k, p);
-        y[p] = v;
-        acc += x[p] * v;
-    }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-// x += alpha p; r -= alpha Ap; block partial sums of r . r
-__global__ void k_update_xr_dot(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                                const double *__restrict__ Ap, const double *__restrict__ scal, size_t n,
-                                double *__restrict__ partial) {
-    __shared__ double sh[256];
-    const double a = scal[S_ALPHA];
-    double acc = 0;
-    GRID_LOOP(k, n) {
-        x[k] += a * p[k];
-        const double v = r[k] - a * Ap[k];
-        r[k] = v;
-        acc += v * v;
-    }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-// fixed-order sum of nb block partials into scal[slot], then an optional
-// scalar step: 1 alpha = rz / pAp, 2 beta = rz_new / rz
+// fixed-order sum of nb block partials 
 __device__ __forceinline__ double block_sum_partials(const double *__restrict__ partial, int nb) {
     __shared__ double sh[kRedBlocks];
     for (int t = threadIdx.x; t < kRedBlocks; t += blockDim.x) sh[t] = t < nb ? partial[t] : 0.0;
@@ -594,32 +296,6 @@ __device__ __forceinline__ double block_sum_partials(const double *__restrict__ 
         __syncthreads();
     }
     return sh[0];
-}
-
-__global__ void k_final(const double *__restrict__ partial, int nb, double *__restrict__ scal, int slot, int step) {
-    const double v = block_sum_partials(partial, nb);
-    if (threadIdx.x == 0) {
-        scal[slot] = v;
-        if (step == 1) scal[S_ALPHA] = scal[S_RZ] / v;
-        if (step == 2) {
-            scal[S_BETA] = v / scal[S_RZ];
-            scal[S_RZ] = v;
-        }
-    }
-}
-
-// sum of r . r, then the loop decision of the CG iteration
-__global__ void k_final_check(const double *__restrict__ partial, int nb, double *__restrict__ scal, int maxit,
-                              DevStats *st, int *flag, cudaGraphConditionalHandle h) {
-    const double rr = block_sum_partials(partial, nb);
-    if (threadIdx.x == 0) {
-        scal[S_RR] = rr;
-        const int it = ++st->pcg_it;
-        st->lin += 1;
-        const bool finite = isfinite(rr);
-        if (!finite) atomicOr(flag, kFlagOverflow);
-        cudaGraphSetConditional(h, (finite && rr > scal[S_TGT] && it < maxit) ? 1u : 0u);
-    }
 }
 
 // Nernst-Planck current of one species through every z face (Sec 2.1, 3.1):
@@ -683,10 +359,9 @@ __global__ void k_eq_rhs(Op A, PhysConst c, EqConst e, const double *__restrict_
                          const double *__restrict__ rho_f, double *__restrict__ rhs, double *__restrict__ dg,
                          int *__restrict__ flag) {
     const size_t n = (size_t)c.nx * c.ny * c.nz;
-    const size_t plane = (size_t)c.nx * c.ny;
     bool bad = false;
     GRID_LOOP(p, n) {
-        const int i = p % A.nx, j = (p / A.nx) % A.ny, k = p / plane;
+        const Pt t = pt_flat(A, (unsigned)p);
         double ch = rho_f ? rho_f[p] : 0.0, sc = 0.0;
         for (int a = 0; a < e.s; ++a) {
             const double r = e.cb[a] * exp(-(mu[a * n + p] + e.q[a] * phi[p]));
@@ -694,9 +369,9 @@ __global__ void k_eq_rhs(Op A, PhysConst c, EqConst e, const double *__restrict_
             sc += (double)(e.q[a] * e.q[a]) * r;
         }
         double b = 4.0 * M_PI * c.lB * ch;
-        if (k == 0) b += c.phi_lo;
-        if (k + 1 == c.nz) b += c.phi_hi;
-        const double v = b - (op_diag(A, i, j, k, p) * phi[p] - op_nbr(A, phi, i, j, k, p));
+        if (t.k == 0) b += c.phi_lo;
+        if (t.k + 1 == c.nz) b += c.phi_hi;
+        const double v = b - (__dmul_rn(op_diag(A, t), phi[p]) - op_nbr(A, phi, phi, t));
         const double d = 4.0 * M_PI * c.lB * sc;
         rhs[p] = v;
         dg[p] = d;
@@ -735,31 +410,6 @@ __global__ void k_eq_update(size_t n, EqConst e, double *__restrict__ phi, const
 
 // ---------------------------------------------------------------------------
 // loop control on the device (conditional graph nodes)
-
-// start of a linear solve: target = tol^2 ||b||^2; enter the loop unless the
-// warm start already meets it
-__global__ void k_pcg_init(double *scal, double tol, DevStats *st, int *flag, cudaGraphConditionalHandle h) {
-    if (!(tol > 0)) tol = st->lin_tol;      // adaptive: set by the Gummel loop
-    double bb = scal[S_BB];
-    if (!(bb > 0)) bb = 1.0;
-    const double tgt = tol * tol * bb;
-    const double rr = scal[S_RR];
-    scal[S_TGT] = tgt;
-    st->pcg_it = 0;
-    const bool finite = isfinite(rr);
-    if (!finite) atomicOr(flag, kFlagOverflow);
-    cudaGraphSetConditional(h, (finite && rr > tgt) ? 1u : 0u);
-}
-
-// end of a CG iteration: continue while ||r||^2 > target and below maxit
-__global__ void k_pcg_check(const double *scal, int maxit, DevStats *st, int *flag, cudaGraphConditionalHandle h) {
-    const double rr = scal[S_RR];
-    const int it = ++st->pcg_it;
-    st->lin += 1;
-    const bool finite = isfinite(rr);
-    if (!finite) atomicOr(flag, kFlagOverflow);
-    cudaGraphSetConditional(h, (finite && rr > scal[S_TGT] && it < maxit) ? 1u : 0u);
-}
 
 // end of a Gummel iteration: residual, status, continue or stop
 __global__ void k_gummel_check(const unsigned long long *dmax, const int *flag, double tol, int max_iter,
@@ -1093,50 +743,135 @@ __global__ void k_phase_mark(double *rec, int slot) {
 // host orchestration
 static int grid_for(size_t n) { return (int)std::min<size_t>(std::max<size_t>((n + 255) / 256, 1), 152 * 16); }
 
-static Op op_of(const Level &L, bool shift = false) {
-    return Op{L.nx, L.ny, L.nz, L.cx, L.cy, L.cz, L.czlo, shift ? L.dg : nullptr};
-}
+static int dot_blocks(size_t n) { return (int)std::min<size_t>(kDotBlocks, (n + 255) / 256); }
+static int blocks_for(size_t n, int threads) { return (int)((n + threads - 1) / threads); }
 
-// one V(1,1) cycle for level l: x = M b (x, b default to the level's vectors)
-static void vcycle(GummelState *g, int l, cudaStream_t st, double *x = nullptr, const double *b = nullptr) {
-    Level &L = g->lv[l];
-    if (!x) x = L.x;
-    if (!b) b = L.b;
-    const Op A = op_of(L, g->shift);
-    const int G = grid_for(L.n);
-    if (l + 1 == (int)g->lv.size()) {
-        if (L.n <= (size_t)kCoarseMax)
-            k_coarse_smem<<<1, 256, 7 * L.n * sizeof(double), st>>>(A, x, b);
-        else
-            k_coarse_solve<<<1, 512, 0, st>>>(A, x, b);
-        return;
+// kernel arguments of the tail's levels, with the operator current at the time
+// of the capture
+static TailArgs tail_args(const GummelState *g, bool shift, const double *b, double *x) {
+    TailArgs a{};
+    a.nl = (int)g->lv.size() - g->lt;
+    unsigned off = 0;
+    for (int l = 0; l < a.nl; ++l) {
+        const Level &L = g->lv[g->lt + l];
+        TailLevel &c = a.lv[l];
+        c.A = op_of(L, shift);
+        c.fx = L.fx; c.fy = L.fy; c.fz = L.fz;
+        c.dfx = FastDiv(L.fx);
+        c.dfy = FastDiv(L.fy);
+        c.dfz = FastDiv(L.fz);
+        c.off = off;
+        c.cx = L.cx; c.cy = L.cy; c.cz = L.cz; c.czlo = L.czlo;
+        c.dg = L.dg; c.dgn = L.dgn; c.idg = L.idg;
+        if (l + 1 < a.nl) off += (unsigned)tail_level_bytes(c.A.nt);
     }
-    Level &C = g->lv[l + 1];
-    // V(2,2): red, black, red, black before; black, red, black, red after
-    k_sweep_zero<<<G, 256, 0, st>>>(A, x, b);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 1);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 0);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 1);
-    k_residual_restrict<<<grid_for(C.n), 256, 0, st>>>(A, x, b, L.fx, L.fy, L.fz, C.nx, C.ny, C.nz, C.b);
-    vcycle(g, l + 1, st);
-    k_prolong_add<<<G, 256, 0, st>>>(x, L.nx, L.ny, L.nz, L.fx, L.fy, L.fz, C.nx, C.ny, C.x, kCoarseScale);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 1);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 0);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 1);
-    k_color_sweep<<<G, 256, 0, st>>>(A, x, b, 0);
+    a.b = b;
+    a.x = x;
+    a.off_coarse = off;
+    return a;
 }
 
-static void coarsen_all(GummelState *g, cudaStream_t st) {
-    for (size_t l = 0; l + 1 < g->lv.size(); ++l) {
+// Which levels the one-CTA tail takes: those from the first of at most
+// kTailMaxPoints points down, as far as shared memory holds them, if the
+// coarsest level fits a warp; otherwise none, and the coarsest level runs its
+// sweeps in a CTA of its own.
+static void plan_tail(GummelState *g) {
+    const int last = (int)g->lv.size() - 1;
+    g->tail = false;
+    g->lt = last;
+    if (g->lv[last].n > (size_t)kCoarseWarp) return;
+    size_t need = sizeof(double) * kCoarseWarp;
+    g->tail = true;
+    g->tail_smem = need;
+    for (int l = last - 1; l >= 0 && last - l < kTailMaxLevels; --l) {
+        const unsigned nt = op_of(g->lv[l]).nt;
+        need += tail_level_bytes(nt);
+        if (g->lv[l].n > (size_t)kTailMaxPoints || nt > (unsigned)(kTailOwn * kTailThreads) || need > kTailSmemMax)
+            break;
+        g->lt = l;
+        g->tail_smem = need;
+    }
+}
+
+// Coarse operators (faces if `faces`, else only the extra diagonal) and the
+// diagonals of every level for the operator now on level 0.
+static void op_setup(GummelState *g, bool faces, cudaStream_t st) {
+    const int last = (int)g->lv.size() - 1;
+    const bool shift = g->shift;
+    for (int l = 0; l < g->lt; ++l) {
         Level &F = g->lv[l], &C = g->lv[l + 1];
-        k_coarsen<<<grid_for(C.n), 256, 0, st>>>(op_of(F), F.fx, F.fy, F.fz, C.nx, C.ny, C.nz, C.cx, C.cy, C.cz,
-                                                 C.czlo);
+        const Op f = op_of(F, shift), c = op_of(C, shift);
+        if (faces)
+            k_coarsen<<<blocks_for(C.n, 128), 128, 0, st>>>(f, F.fx, F.fy, F.fz, c, C.cx, C.cy, C.cz, C.czlo);
+        if (shift)
+            k_restrict<<<blocks_for(C.n, 128), 128, 0, st>>>(f, F.dg, F.fx, F.fy, F.fz, c, C.dg);
     }
+    for (int l = 0; l < (g->tail ? g->lt + 1 : last + 1); ++l) {
+        Level &L = g->lv[l];
+        k_diag<<<blocks_for(L.n, 128), 128, 0, st>>>(op_of(L, shift), L.dgn, L.idg);
+    }
+    if (g->tail && g->lt < last)
+        k_tail_setup<<<1, kTailThreads, 0, st>>>(tail_args(g, shift, nullptr, nullptr), faces ? 1 : 0);
 }
 
-static void dot(GummelState *g, const double *a, const double *b, size_t n, int slot, cudaStream_t st) {
-    k_dot_partial<<<kRedBlocks, 256, 0, st>>>(a, b, n, g->partial);
-    k_dot_final<<<1, 256, 0, st>>>(g->partial, g->scal, slot);
+// x = M b, one V(2,2) cycle on the current operator, from the start values
+// that the kernel producing b left in x (red: b / diag, black: 0).  On level 0
+// x = z, b = r, and the block sums of b . x go to `part`; returns their number.
+static int vcycle(GummelState *g, cudaStream_t st, double *part) {
+    const int last = (int)g->lv.size() - 1;
+    auto xof = [&](int l) { return l ? g->lv[l].x : g->z; };
+    auto x2of = [&](int l) { return l ? g->lv[l].x2 : g->z2; };
+    auto bof = [&](int l) { return l ? (const double *)g->lv[l].b : (const double *)g->r; };
+    const size_t n0 = g->lv[0].n;
+    const int nb = dot_blocks(n0);
+    for (int l = 0; l < g->lt; ++l) {
+        Level &L = g->lv[l], &C = g->lv[l + 1];
+        const Op A = op_of(L, g->shift);
+        const int G = blocks_for(A.nt, kSweepThreads);
+        double *x = xof(l), *y = x2of(l);
+        const double *b = bof(l);
+        // odd levels: red starts in y, black in x; every sweep writes the
+        // buffer its colour is not in, and all end in x
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, x, y, b, 1);
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, y, x, b, 0);
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, y, x, b, 1);
+        const size_t sm = sizeof(double) * kRestrictCells * L.fx * L.fy * L.fz;
+        k_residual_restrict<<<blocks_for(C.n, kRestrictCells), 256, sm, st>>>(
+            A, x, b, L.fx, L.fy, L.fz, op_of(C, g->shift), C.b, C.x2, C.x);
+    }
+    if (g->tail) {
+        k_tail<<<1, kTailThreads, g->tail_smem, st>>>(tail_args(g, g->shift, bof(g->lt), xof(g->lt)));
+    } else {
+        Level &L = g->lv[last];
+        const Op A = op_of(L, g->shift);
+        if (L.n <= (size_t)kCoarseMax)
+            k_coarse_smem<<<1, 256, 7 * L.n * sizeof(double), st>>>(A, xof(last), bof(last));
+        else
+            k_coarse_solve<<<1, 512, 0, st>>>(A, xof(last), bof(last));
+    }
+    // the last red sweep of level 0 carries the dot product while a slot holds
+    // one point; longer slots are summed apart (with 512 CTAs for 152 SMs the
+    // sweep would lose more than the launch costs)
+    const bool fuse_dot = g->lt > 0 && n0 <= (size_t)kDotBlocks * 256 && g->lv[0].nx % 2 == 0;
+    for (int l = g->lt - 1; l >= 0; --l) {
+        Level &L = g->lv[l], &C = g->lv[l + 1];
+        const Op A = op_of(L, g->shift);
+        const int G = blocks_for(A.nt, kSweepThreads);
+        double *x = xof(l), *y = x2of(l);
+        const double *b = bof(l);
+        k_prolong_add<<<G, kSweepThreads, 0, st>>>(A, x, FastDiv(L.fx), FastDiv(L.fy), FastDiv(L.fz), C.nx, C.ny, C.x,
+                                                   kCoarseScale);
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, x, y, b, 1);
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, x, y, b, 0);
+        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, y, x, b, 1);
+        if (l > 0 || !fuse_dot) {
+            k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, y, x, b, 0);
+        } else {
+            k_sweep_dot<<<nb, 128, 0, st>>>(A, x, y, x, b, part);
+        }
+    }
+    if (!fuse_dot) k_dot<<<nb, 256, 0, st>>>(g->r, g->z, (unsigned)n0, part);
+    return nb;
 }
 
 // Append a conditional WHILE node to the capture on `st`; later captured work
@@ -1165,24 +900,19 @@ static cudaError_t add_while(cudaStream_t st, unsigned dflt, cudaGraphConditiona
     return cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
-// MG-preconditioned CG on level 0's operator, recorded into the capture on
-// `st` with the iteration loop as a conditional WHILE node whose body is
-// captured on `sb`.  x holds the initial guess; stops at ||r||_2 <= tol ||b||_2
-// or maxit iterations.  All reductions have a fixed shape.
+// MG-preconditioned CG on level 0's operator (after op_setup), recorded into
+// the capture on `st` with the iteration loop as a conditional WHILE node
+// whose body is captured on `sb`.  x holds the initial guess; stops at
+// ||r||_2 <= tol ||b||_2 or maxit iterations.  All reductions have a fixed
+// shape.
 static cudaError_t pcg_capture(GummelState *g, double *x, const double *b, double tol, int maxit, int *flag,
                                cudaStream_t st, cudaStream_t sb) {
-    Level &L0 = g->lv[0];
-    const Op A = op_of(L0, g->shift);
-    const size_t n = L0.n;
-    const int G = grid_for(n);
-    const int NB = std::min(G, kRedBlocks);
-    double *r = g->r, *z = g->z, *p = g->pv, *Ap = g->Ap;
-    dot(g, b, b, n, S_BB, st);
-    k_residual<<<G, 256, 0, st>>>(A, x, b, r);
-    dot(g, r, r, n, S_RR, st);
-    vcycle(g, 0, st, z, r);
-    k_copy<<<G, 256, 0, st>>>(p, z, n);
-    dot(g, r, z, n, S_RZ, st);
+    const Op A = op_of(g->lv[0], g->shift);
+    const int NB = dot_blocks(A.n);
+    double *r = g->r, *z = g->z, *z2 = g->z2, *p = g->pv, *Ap = g->Ap;
+    double *part_bb = g->partial, *part_rr = part_bb + kDotBlocks, *part_rz = part_rr + kDotBlocks,
+           *part_pap = part_rz + kDotBlocks;
+    k_pcg_start<<<NB, 256, 0, st>>>(A, x, b, r, z2, z, part_bb, part_rr);
     cudaStreamCaptureStatus cs;
     cudaGraph_t cg = nullptr;
     cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &cg, nullptr, nullptr, nullptr);
@@ -1190,36 +920,17 @@ static cudaError_t pcg_capture(GummelState *g, double *x, const double *b, doubl
     cudaGraphConditionalHandle h;
     e = cudaGraphConditionalHandleCreate(&h, cg, 0, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return e;
-    k_pcg_init<<<1, 1, 0, st>>>(g->scal, tol, g->stats, flag, h);
+    k_pcg_init<<<1, 128, 0, st>>>(g->scal, part_bb, part_rr, NB, tol, g->stats, flag, h);
     cudaGraph_t body = nullptr;
-    {
-        const cudaGraphNode_t *deps = nullptr;
-        const cudaGraphEdgeData *ed = nullptr;
-        size_t nd = 0;
-        e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &cg, &deps, &ed, &nd);
-        if (e != cudaSuccess) return e;
-        cudaGraphNodeParams prm = {};
-        prm.type = cudaGraphNodeTypeConditional;
-        prm.conditional.handle = h;
-        prm.conditional.type = cudaGraphCondTypeWhile;
-        prm.conditional.size = 1;
-        cudaGraphNode_t node;
-        e = cudaGraphAddNode(&node, cg, deps, ed, nd, &prm);
-        if (e != cudaSuccess) return e;
-        body = prm.conditional.phGraph_out[0];
-        e = cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
-        if (e != cudaSuccess) return e;
-    }
+    e = add_while(st, 0, &h, &body, true);
+    if (e != cudaSuccess) return e;
     e = cudaStreamBeginCaptureToGraph(sb, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return e;
-    k_apply_dot<<<NB, 256, 0, sb>>>(A, p, Ap, g->partial);
-    k_final<<<1, 256, 0, sb>>>(g->partial, NB, g->scal, S_PAP, 1);
-    k_update_xr_dot<<<NB, 256, 0, sb>>>(x, r, p, Ap, g->scal, n, g->partial);
-    k_final_check<<<1, 256, 0, sb>>>(g->partial, NB, g->scal, maxit, g->stats, flag, h);
-    vcycle(g, 0, sb, z, r);
-    k_dot_partial<<<NB, 256, 0, sb>>>(r, z, n, g->partial);
-    k_final<<<1, 256, 0, sb>>>(g->partial, NB, g->scal, S_RZNEW, 2);
-    k_update_p<<<G, 256, 0, sb>>>(p, z, g->scal, n);
+    const int nrz = vcycle(g, sb, part_rz);
+    k_pcg_direction<<<NB, 256, 0, sb>>>(p, z, g->scal, part_rz, nrz, g->stats, A.n);
+    k_pcg_apply<<<NB, 256, 0, sb>>>(A, p, Ap, part_pap);
+    k_pcg_update<<<NB, 256, 0, sb>>>(A, x, r, p, Ap, z2, z, g->scal, part_pap, NB, g->stats, part_rr);
+    k_pcg_check<<<1, 128, 0, sb>>>(g->scal, part_rr, NB, maxit, g->stats, flag, h);
     return cudaStreamEndCapture(sb, &body);
 }
 
@@ -1257,25 +968,32 @@ int gummel_setup(Problem *p) {
         L.fz = fac(nz);
         bool last = L.n <= 8 || (L.fx == 1 && L.fy == 1 && L.fz == 1) || g->lv.size() >= 16;
         if (last) L.fx = L.fy = L.fz = 1;
+        L.odd = (p->bc[0] == PNP_BC_PERIODIC && nx % 2) || (p->bc[1] == PNP_BC_PERIODIC && ny % 2);
         g->lv.push_back(L);
         if (last) break;
         nx /= L.fx; ny /= L.fy; nz /= L.fz;
     }
-    // coarsest must fit the single-CTA solver comfortably
+    plan_tail(g);
     const size_t N = p->npts();
     bool ok = true;
     for (size_t l = 0; l < g->lv.size() && ok; ++l) {
         Level &L = g->lv[l];
-        ok = alloc(&L.cx, L.n) && alloc(&L.cy, L.n) && alloc(&L.cz, L.n) && alloc(&L.czlo, L.n) &&
-             alloc(&L.pcx, L.n) && alloc(&L.pcy, L.n) && alloc(&L.pcz, L.n) && alloc(&L.pczlo, L.n) &&
-             alloc(&L.x, L.n) && alloc(&L.b, L.n) && alloc(&L.r, L.n);
+        const size_t plane = (size_t)L.nx * L.ny;
+        ok = alloc(&L.cx, L.n) && alloc(&L.cy, L.n) && alloc(&L.cz, L.n) && alloc(&L.czlo, plane) &&
+             alloc(&L.pcx, L.n) && alloc(&L.pcy, L.n) && alloc(&L.pcz, L.n) && alloc(&L.pczlo, plane) &&
+             alloc(&L.dgn, L.n) && alloc(&L.idg, L.n);
+        if (ok && l > 0) ok = alloc(&L.x, L.n) && alloc(&L.b, L.n);   // level 0 works on z and r
+        L.x2 = L.x;
+        if (ok && l > 0 && L.odd) ok = alloc(&L.x2, L.n);
         L.dg = nullptr;
         if (ok && (p->eq_init || p->screened)) ok = alloc(&L.dg, L.n);
     }
     ok = ok && alloc(&g->mu, N * p->s) && alloc(&g->phi, N) && alloc(&g->rho, N * p->s) &&
          alloc(&g->rhs, N) && alloc(&g->x, N) && alloc(&g->r, N) &&
-         alloc(&g->z, N) && alloc(&g->pv, N) && alloc(&g->Ap, N) && alloc(&g->partial, kRedBlocks) &&
-         alloc(&g->scal, S_COUNT);
+         alloc(&g->z, N) && alloc(&g->pv, N) && alloc(&g->Ap, N) && alloc(&g->em, N) &&
+         alloc(&g->partial, 4 * kDotBlocks) && alloc(&g->scal, S_COUNT);
+    g->z2 = g->z;
+    if (ok && g->lv[0].odd) ok = alloc(&g->z2, N);
     if (ok && p->rho_mix == PNP_MIX_ADAPTIVE) ok = alloc(&g->lam, N * p->s) && alloc(&g->prev, N * p->s);
     if (ok && p->phase_timing) ok = alloc(&g->phase, kPhases + 1);
     if (ok && p->aa_depth > 0) {
@@ -1298,12 +1016,13 @@ int gummel_setup(Problem *p) {
     }
     p->device_bytes += g->bytes;
     p->mg_levels = (int)g->lv.size();
+    cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
     cudaFuncSetAttribute(k_coarse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, 7 * kCoarseMax * 8);
     // Poisson operator on every level (into the p* arrays)
     PhysConst c{p->nx, p->ny, p->nz, p->bc[0], p->bc[1], p->lB, p->phi_lo, p->phi_hi};
     set_operator(g, true);
     k_poisson_coefs<<<grid_for(N), 256, 0, p->stream>>>(c, g->lv[0].cx, g->lv[0].cy, g->lv[0].cz, g->lv[0].czlo);
-    coarsen_all(g, p->stream);
+    op_setup(g, true, p->stream);
     set_operator(g, true);
     const int rc = cuda_status(cudaStreamSynchronize(p->stream));
     if (rc) gummel_free(p);
@@ -1314,14 +1033,16 @@ void gummel_free(Problem *p) {
     GummelState *g = p->gs;
     if (!g) return;
     for (auto &L : g->lv) {
-        for (double *a : {L.cx, L.cy, L.cz, L.czlo, L.pcx, L.pcy, L.pcz, L.pczlo, L.dg, L.x, L.b, L.r})
+        for (double *a : {L.cx, L.cy, L.cz, L.czlo, L.pcx, L.pcy, L.pcz, L.pczlo, L.dg, L.dgn, L.idg, L.x, L.b})
             dfree(a, p->stream);
+        if (L.x2 != L.x) dfree(L.x2, p->stream);
     }
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
     for (int k = 0; k < 2; ++k)
         if (g->cap[k]) cudaStreamDestroy(g->cap[k]);
-    for (double *a : {g->mu, g->phi, g->rho, g->rhs, g->x, g->r, g->z, g->pv, g->Ap, g->partial, g->scal, g->lam,
+    if (g->z2 != g->z) dfree(g->z2, p->stream);
+    for (double *a : {g->mu, g->phi, g->rho, g->rhs, g->x, g->r, g->z, g->pv, g->Ap, g->em, g->partial, g->scal, g->lam,
                       g->prev, g->aa_X, g->aa_F, g->aa_part, g->aa_xb, g->aa_fb, g->phase})
         dfree(a, p->stream);
     dfree(g->aa, p->stream);
@@ -1383,12 +1104,9 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             set_operator(g, true);
             Level &L0 = g->lv[0];
             k_eq_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, ec, g->phi, g->mu, d_rhof, g->rhs, L0.dg, p->d_flag);
-            for (size_t l = 0; l + 1 < g->lv.size(); ++l) {
-                Level &F = g->lv[l], &C = g->lv[l + 1];
-                k_restrict<<<grid_for(C.n), 256, 0, sb>>>(F.dg, F.nx, F.ny, F.fx, F.fy, F.fz, C.nx, C.ny, C.nz, C.dg);
-            }
             k_fill<<<G, 256, 0, sb>>>(g->x, 0.0, N);
             g->shift = true;
+            op_setup(g, false, sb);
             e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
             g->shift = false;
             set_operator(g, true);
@@ -1423,12 +1141,9 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             // (A + dg) dphi = b(rho) - A phi, phi* = phi + dphi
             Level &L0 = g->lv[0];
             k_scr_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, g->rho, s, d_q, d_rhof, g->phi, g->rhs, L0.dg);
-            for (size_t l = 0; l + 1 < g->lv.size(); ++l) {
-                Level &F = g->lv[l], &C = g->lv[l + 1];
-                k_restrict<<<grid_for(C.n), 256, 0, sb>>>(F.dg, F.nx, F.ny, F.fx, F.fy, F.fz, C.nx, C.ny, C.nz, C.dg);
-            }
             k_fill<<<G, 256, 0, sb>>>(g->x, 0.0, N);
             g->shift = true;
+            op_setup(g, false, sb);
             e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
             g->shift = false;
             set_operator(g, true);
@@ -1436,6 +1151,7 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
         } else {
             k_poisson_rhs<<<G, 256, 0, sb>>>(c, g->rho, s, d_q, d_rhof, g->rhs);
             k_copy<<<G, 256, 0, sb>>>(g->x, g->phi, N);
+            op_setup(g, false, sb);
             e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
             set_operator(g, true);
             k_relax_phi<<<G, 256, 0, sb>>>(g->phi, g->x, p->lambda_phi, N, g->dmax);
@@ -1451,12 +1167,13 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             nc.rlo = p->rho_b[i] * std::exp(p->q[i] * p->phi_lo + p->mu_bulk[i]);
             nc.rhi = p->rho_b[i] * std::exp(p->q[i] * p->phi_hi + p->mu_bulk[i]);
             Level &L0 = g->lv[0];
-            k_np_setup<<<G, 256, 0, sb>>>(c, nc, g->phi, g->mu + i * N, g->rho + i * N, L0.cx, L0.cy, L0.cz,
-                                          L0.czlo, g->rhs, g->x, p->d_flag);
-            coarsen_all(g, sb);
+            const Op A0 = op_of(L0);
+            k_np_mobility<<<G, 256, 0, sb>>>(N, nc, g->phi, g->mu + i * N, g->rho + i * N, g->em, g->x, p->d_flag);
+            k_np_faces<<<blocks_for(N, 128), 128, 0, sb>>>(c, nc, A0, g->em, L0.cx, L0.cy, L0.cz, L0.czlo, g->rhs);
+            op_setup(g, true, sb);
             e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
-            k_np_finish<<<G, 256, 0, sb>>>(N, (double)p->q[i], p->lambda_rho, p->rho_mix, 1.0 / p->rho_b[i], g->phi,
-                                           g->mu + i * N, g->x, g->rho + i * N, g->lam ? g->lam + i * N : nullptr,
+            k_np_finish<<<G, 256, 0, sb>>>(N, p->lambda_rho, p->rho_mix, 1.0 / p->rho_b[i], g->em,
+                                           g->x, g->rho + i * N, g->lam ? g->lam + i * N : nullptr,
                                            g->prev ? g->prev + i * N : nullptr, g->dmax, p->d_flag);
         }
         if (g->phase) k_phase_mark<<<1, 1, 0, sb>>>(g->phase, 2);
