@@ -28,10 +28,8 @@ namespace pnp {
 struct DevStats {
     int status;            // PNP_OK, PNP_ERR_NOT_CONVERGED, PNP_ERR_PACKING, PNP_ERR_OVERFLOW
     int iters;             // Gummel iterations done
-    int pcg_it;            // iterations of the current linear solve
-    int pad;
     double residual;       // last Gummel residual
-    long long lin;         // linear iterations over the solve
+    unsigned long long lin;    // linear iterations over the solve
     double lin_tol;        // current tolerance of the linear solves (adaptive mode)
     int eq_enable;         // run the equilibrium stage (set before each launch)
     int eq_iters;          // its iterations
@@ -62,25 +60,36 @@ constexpr int kAaBacktrack = 8;    // step halvings after the restart from the p
 
 namespace pnp {
 
-struct GummelState {
+// Everything one linear solve works on.  Lane 0 solves the Poisson equation
+// and owns its memory; the Nernst-Planck solves of an iteration depend only on
+// phi and mu_ex, not on one another, so species i runs on lane i % lanes and
+// the lanes run side by side (build_graph).
+struct Lane {
     std::vector<Level> lv;
     int lt = 0;                    // first level of the one-CTA tail (or the coarsest, without one)
     bool tail = false;
     size_t tail_smem = 0;
+    double *rhs = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *pv = nullptr, *Ap = nullptr;
+    double *z2 = nullptr;          // second buffer of z on odd grids (z otherwise)
+    double *em = nullptr;          // exp(-(q phi + mu)) of the current species
+    double *partial = nullptr;     // four sets of kDotBlocks partial sums
+    LinCtl *ctl = nullptr;
+    bool shift = false;            // operators carry the levels' dg while capturing
+};
+
+struct GummelState {
+    std::vector<Lane> lane;
     double *mu = nullptr;
     double *phi = nullptr, *rho = nullptr;    // solve state the graph works on
     DevStats *stats = nullptr;
     int *keep_q = nullptr;                    // valences and fixed charge used by the graph
     double *keep_rhof = nullptr;
     cudaStream_t cap[2] = {nullptr, nullptr}; // capture streams of the loop bodies
+    std::vector<cudaStream_t> fork;           // and of the branches inside one
+    std::vector<cudaEvent_t> ev;              // branch points
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    double *rhs = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *pv = nullptr, *Ap = nullptr;
-    double *z2 = nullptr;          // second buffer of z on odd grids (z otherwise)
-    double *em = nullptr;          // exp(-(q phi + mu)) of the current species
-    double *partial = nullptr;     // four sets of kDotBlocks partial sums
     double *lam = nullptr, *prev = nullptr;   // PNP_MIX_ADAPTIVE: per-point factor and last step
-    double *scal = nullptr;        // device scalars
     // Anderson mixing (depth m > 0): history of m + 1 iterates x = (phi, ln rho)
     // and residuals f = G(x) - x, [m+1][(1+s) N] each, a control block and the
     // Gram reduction's block partials
@@ -90,7 +99,6 @@ struct GummelState {
     double *phase = nullptr;          // PNP_FLAG_PHASE_TIMING: ns per phase, then the last mark
     unsigned long long *dmax = nullptr;
     size_t bytes = 0;
-    bool shift = false;            // operators carry the levels' dg while capturing
 };
 
 constexpr int kRedBlocks = 512;
@@ -468,7 +476,6 @@ __global__ void k_stats_reset(DevStats *st, int eq_enable) {
     st->lin_tol = 1e-6;
     st->status = PNP_ERR_NOT_CONVERGED;
     st->iters = 0;
-    st->pcg_it = 0;
     st->residual = 0;
     st->lin = 0;
     st->eq_enable = eq_enable;
@@ -748,7 +755,7 @@ static int blocks_for(size_t n, int threads) { return (int)((n + threads - 1) / 
 
 // kernel arguments of the tail's levels, with the operator current at the time
 // of the capture
-static TailArgs tail_args(const GummelState *g, bool shift, const double *b, double *x) {
+static TailArgs tail_args(const Lane *g, bool shift, const double *b, double *x) {
     TailArgs a{};
     a.nl = (int)g->lv.size() - g->lt;
     unsigned off = 0;
@@ -775,7 +782,7 @@ static TailArgs tail_args(const GummelState *g, bool shift, const double *b, dou
 // kTailMaxPoints points down, as far as shared memory holds them, if the
 // coarsest level fits a warp; otherwise none, and the coarsest level runs its
 // sweeps in a CTA of its own.
-static void plan_tail(GummelState *g) {
+static void plan_tail(Lane *g) {
     const int last = (int)g->lv.size() - 1;
     g->tail = false;
     g->lt = last;
@@ -795,7 +802,7 @@ static void plan_tail(GummelState *g) {
 
 // Coarse operators (faces if `faces`, else only the extra diagonal) and the
 // diagonals of every level for the operator now on level 0.
-static void op_setup(GummelState *g, bool faces, cudaStream_t st) {
+static void op_setup(Lane *g, bool faces, cudaStream_t st) {
     const int last = (int)g->lv.size() - 1;
     const bool shift = g->shift;
     for (int l = 0; l < g->lt; ++l) {
@@ -817,7 +824,7 @@ static void op_setup(GummelState *g, bool faces, cudaStream_t st) {
 // x = M b, one V(2,2) cycle on the current operator, from the start values
 // that the kernel producing b left in x (red: b / diag, black: 0).  On level 0
 // x = z, b = r, and the block sums of b . x go to `part`; returns their number.
-static int vcycle(GummelState *g, cudaStream_t st, double *part) {
+static int vcycle(Lane *g, cudaStream_t st, double *part) {
     const int last = (int)g->lv.size() - 1;
     auto xof = [&](int l) { return l ? g->lv[l].x : g->z; };
     auto x2of = [&](int l) { return l ? g->lv[l].x2 : g->z2; };
@@ -905,8 +912,8 @@ static cudaError_t add_while(cudaStream_t st, unsigned dflt, cudaGraphConditiona
 // whose body is captured on `sb`.  x holds the initial guess; stops at
 // ||r||_2 <= tol ||b||_2 or maxit iterations.  All reductions have a fixed
 // shape.
-static cudaError_t pcg_capture(GummelState *g, double *x, const double *b, double tol, int maxit, int *flag,
-                               cudaStream_t st, cudaStream_t sb) {
+static cudaError_t pcg_capture(Lane *g, double *x, const double *b, double tol, int maxit, int *flag,
+                               DevStats *stats, cudaStream_t st, cudaStream_t sb) {
     const Op A = op_of(g->lv[0], g->shift);
     const int NB = dot_blocks(A.n);
     double *r = g->r, *z = g->z, *z2 = g->z2, *p = g->pv, *Ap = g->Ap;
@@ -920,21 +927,21 @@ static cudaError_t pcg_capture(GummelState *g, double *x, const double *b, doubl
     cudaGraphConditionalHandle h;
     e = cudaGraphConditionalHandleCreate(&h, cg, 0, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return e;
-    k_pcg_init<<<1, 128, 0, st>>>(g->scal, part_bb, part_rr, NB, tol, g->stats, flag, h);
+    k_pcg_init<<<1, 128, 0, st>>>(g->ctl, part_bb, part_rr, NB, tol, stats, flag, h);
     cudaGraph_t body = nullptr;
     e = add_while(st, 0, &h, &body, true);
     if (e != cudaSuccess) return e;
     e = cudaStreamBeginCaptureToGraph(sb, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return e;
     const int nrz = vcycle(g, sb, part_rz);
-    k_pcg_direction<<<NB, 256, 0, sb>>>(p, z, g->scal, part_rz, nrz, g->stats, A.n);
+    k_pcg_direction<<<NB, 256, 0, sb>>>(p, z, g->ctl, part_rz, nrz, A.n);
     k_pcg_apply<<<NB, 256, 0, sb>>>(A, p, Ap, part_pap);
-    k_pcg_update<<<NB, 256, 0, sb>>>(A, x, r, p, Ap, z2, z, g->scal, part_pap, NB, g->stats, part_rr);
-    k_pcg_check<<<1, 128, 0, sb>>>(g->scal, part_rr, NB, maxit, g->stats, flag, h);
+    k_pcg_update<<<NB, 256, 0, sb>>>(A, x, r, p, Ap, z2, z, g->ctl, part_pap, NB, part_rr);
+    k_pcg_check<<<1, 128, 0, sb>>>(g->ctl, part_rr, NB, maxit, stats, flag, h);
     return cudaStreamEndCapture(sb, &body);
 }
 
-static void set_operator(GummelState *g, bool poisson) {
+static void set_operator(Lane *g, bool poisson) {
     for (auto &L : g->lv) {
         if (poisson) {
             std::swap(L.cx, L.pcx);
@@ -955,6 +962,7 @@ int gummel_setup(Problem *p) {
         return true;
     };
     // levels
+    Lane first;
     int nx = p->nx, ny = p->ny, nz = p->nz;
     while (true) {
         Level L{};
@@ -966,34 +974,55 @@ int gummel_setup(Problem *p) {
         L.fx = fac(nx);
         L.fy = fac(ny);
         L.fz = fac(nz);
-        bool last = L.n <= 8 || (L.fx == 1 && L.fy == 1 && L.fz == 1) || g->lv.size() >= 16;
+        bool last = L.n <= 8 || (L.fx == 1 && L.fy == 1 && L.fz == 1) || first.lv.size() >= 16;
         if (last) L.fx = L.fy = L.fz = 1;
         L.odd = (p->bc[0] == PNP_BC_PERIODIC && nx % 2) || (p->bc[1] == PNP_BC_PERIODIC && ny % 2);
-        g->lv.push_back(L);
+        first.lv.push_back(L);
         if (last) break;
         nx /= L.fx; ny /= L.fy; nz /= L.fz;
     }
-    plan_tail(g);
+    plan_tail(&first);
     const size_t N = p->npts();
-    bool ok = true;
-    for (size_t l = 0; l < g->lv.size() && ok; ++l) {
-        Level &L = g->lv[l];
-        const size_t plane = (size_t)L.nx * L.ny;
-        ok = alloc(&L.cx, L.n) && alloc(&L.cy, L.n) && alloc(&L.cz, L.n) && alloc(&L.czlo, plane) &&
-             alloc(&L.pcx, L.n) && alloc(&L.pcy, L.n) && alloc(&L.pcz, L.n) && alloc(&L.pczlo, plane) &&
-             alloc(&L.dgn, L.n) && alloc(&L.idg, L.n);
-        if (ok && l > 0) ok = alloc(&L.x, L.n) && alloc(&L.b, L.n);   // level 0 works on z and r
-        L.x2 = L.x;
-        if (ok && l > 0 && L.odd) ok = alloc(&L.x2, L.n);
-        L.dg = nullptr;
-        if (ok && (p->eq_init || p->screened)) ok = alloc(&L.dg, L.n);
+    // arrays of a lane by `get` (false: no memory); lane 0 also carries the
+    // Poisson operator
+    auto lane_arrays = [&](Lane &a, bool poisson, auto get) {
+        bool ok = true;
+        for (size_t l = 0; l < a.lv.size() && ok; ++l) {
+            Level &L = a.lv[l];
+            const size_t plane = (size_t)L.nx * L.ny;
+            ok = get(&L.cx, L.n) && get(&L.cy, L.n) && get(&L.cz, L.n) && get(&L.czlo, plane) && get(&L.dgn, L.n) &&
+                 get(&L.idg, L.n);
+            if (ok && poisson)
+                ok = get(&L.pcx, L.n) && get(&L.pcy, L.n) && get(&L.pcz, L.n) && get(&L.pczlo, plane);
+            if (ok && poisson && (p->eq_init || p->screened)) ok = get(&L.dg, L.n);
+            if (ok && l > 0) ok = get(&L.x, L.n) && get(&L.b, L.n);   // level 0 works on z and r
+            L.x2 = L.x;
+            if (ok && l > 0 && L.odd) ok = get(&L.x2, L.n);
+        }
+        ok = ok && get(&a.rhs, N) && get(&a.x, N) && get(&a.r, N) && get(&a.z, N) && get(&a.pv, N) && get(&a.Ap, N) &&
+             get(&a.em, N) && get(&a.partial, 4 * kDotBlocks) && get((double **)&a.ctl, sizeof(LinCtl) / sizeof(double));
+        a.z2 = a.z;
+        if (ok && a.lv[0].odd) ok = get(&a.z2, N);
+        return ok;
+    };
+    g->lane.push_back(first);
+    bool ok = lane_arrays(g->lane[0], true, alloc);
+    // The other lanes live in the mu_ex workspace, which is idle while the
+    // Nernst-Planck systems are solved: as many as fit, at most one per species
+    // (two species need one, about 13 of its 22 or more fields).
+    for (size_t off = 0; ok && g->lane.size() < (size_t)p->s;) {
+        Lane a = first;
+        const bool fits = lane_arrays(a, false, [&](double **ptr, size_t n) {
+            const size_t bytes = (sizeof(double) * std::max<size_t>(n, 1) + 255) / 256 * 256;
+            if (off + bytes > p->work_bytes) return false;
+            *ptr = (double *)((char *)p->d_work + off);
+            off += bytes;
+            return true;
+        });
+        if (!fits) break;
+        g->lane.push_back(a);
     }
-    ok = ok && alloc(&g->mu, N * p->s) && alloc(&g->phi, N) && alloc(&g->rho, N * p->s) &&
-         alloc(&g->rhs, N) && alloc(&g->x, N) && alloc(&g->r, N) &&
-         alloc(&g->z, N) && alloc(&g->pv, N) && alloc(&g->Ap, N) && alloc(&g->em, N) &&
-         alloc(&g->partial, 4 * kDotBlocks) && alloc(&g->scal, S_COUNT);
-    g->z2 = g->z;
-    if (ok && g->lv[0].odd) ok = alloc(&g->z2, N);
+    ok = ok && alloc(&g->mu, N * p->s) && alloc(&g->phi, N) && alloc(&g->rho, N * p->s);
     if (ok && p->rho_mix == PNP_MIX_ADAPTIVE) ok = alloc(&g->lam, N * p->s) && alloc(&g->prev, N * p->s);
     if (ok && p->phase_timing) ok = alloc(&g->phase, kPhases + 1);
     if (ok && p->aa_depth > 0) {
@@ -1007,6 +1036,17 @@ int gummel_setup(Problem *p) {
         if (ok && dmalloc((void **)&g->stats, sizeof(DevStats), p->stream) != cudaSuccess) ok = false;
         for (int k = 0; k < 2 && ok; ++k)
             if (cudaStreamCreateWithFlags(&g->cap[k], cudaStreamNonBlocking) != cudaSuccess) ok = false;
+        // one branch per lane beyond the first, at least one for mu_ex
+        for (size_t k = 0; k < std::max<size_t>(1, g->lane.size() - 1) && ok; ++k) {
+            cudaStream_t b = nullptr;
+            ok = cudaStreamCreateWithFlags(&b, cudaStreamNonBlocking) == cudaSuccess;
+            if (ok) g->fork.push_back(b);
+        }
+        for (size_t k = 0; k < g->fork.size() + 1 && ok; ++k) {
+            cudaEvent_t v = nullptr;
+            ok = cudaEventCreateWithFlags(&v, cudaEventDisableTiming) == cudaSuccess;
+            if (ok) g->ev.push_back(v);
+        }
     }
     if (!ok) {
         // nothing half-built stays behind for a later solve to take as ready
@@ -1015,15 +1055,17 @@ int gummel_setup(Problem *p) {
         return PNP_ERR_NOMEM;
     }
     p->device_bytes += g->bytes;
-    p->mg_levels = (int)g->lv.size();
+    p->mg_levels = (int)first.lv.size();
     cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax);
     cudaFuncSetAttribute(k_coarse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, 7 * kCoarseMax * 8);
     // Poisson operator on every level (into the p* arrays)
     PhysConst c{p->nx, p->ny, p->nz, p->bc[0], p->bc[1], p->lB, p->phi_lo, p->phi_hi};
-    set_operator(g, true);
-    k_poisson_coefs<<<grid_for(N), 256, 0, p->stream>>>(c, g->lv[0].cx, g->lv[0].cy, g->lv[0].cz, g->lv[0].czlo);
-    op_setup(g, true, p->stream);
-    set_operator(g, true);
+    Lane *a = &g->lane[0];
+    Level &L0 = a->lv[0];
+    set_operator(a, true);
+    k_poisson_coefs<<<grid_for(N), 256, 0, p->stream>>>(c, L0.cx, L0.cy, L0.cz, L0.czlo);
+    op_setup(a, true, p->stream);
+    set_operator(a, true);
     const int rc = cuda_status(cudaStreamSynchronize(p->stream));
     if (rc) gummel_free(p);
     return rc;
@@ -1032,18 +1074,24 @@ int gummel_setup(Problem *p) {
 void gummel_free(Problem *p) {
     GummelState *g = p->gs;
     if (!g) return;
-    for (auto &L : g->lv) {
-        for (double *a : {L.cx, L.cy, L.cz, L.czlo, L.pcx, L.pcy, L.pcz, L.pczlo, L.dg, L.dgn, L.idg, L.x, L.b})
-            dfree(a, p->stream);
-        if (L.x2 != L.x) dfree(L.x2, p->stream);
+    if (!g->lane.empty()) {        // the other lanes lie in the workspace
+        Lane &a = g->lane[0];
+        for (auto &L : a.lv) {
+            for (double *v : {L.cx, L.cy, L.cz, L.czlo, L.pcx, L.pcy, L.pcz, L.pczlo, L.dg, L.dgn, L.idg, L.x, L.b})
+                dfree(v, p->stream);
+            if (L.x2 != L.x) dfree(L.x2, p->stream);
+        }
+        if (a.z2 != a.z) dfree(a.z2, p->stream);
+        for (double *v : {a.rhs, a.x, a.r, a.z, a.pv, a.Ap, a.em, a.partial}) dfree(v, p->stream);
+        dfree(a.ctl, p->stream);
     }
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
     for (int k = 0; k < 2; ++k)
         if (g->cap[k]) cudaStreamDestroy(g->cap[k]);
-    if (g->z2 != g->z) dfree(g->z2, p->stream);
-    for (double *a : {g->mu, g->phi, g->rho, g->rhs, g->x, g->r, g->z, g->pv, g->Ap, g->em, g->partial, g->scal, g->lam,
-                      g->prev, g->aa_X, g->aa_F, g->aa_part, g->aa_xb, g->aa_fb, g->phase})
+    for (cudaStream_t b : g->fork) cudaStreamDestroy(b);
+    for (cudaEvent_t v : g->ev) cudaEventDestroy(v);
+    for (double *a : {g->mu, g->phi, g->rho, g->lam, g->prev, g->aa_X, g->aa_F, g->aa_part, g->aa_xb, g->aa_fb, g->phase})
         dfree(a, p->stream);
     dfree(g->aa, p->stream);
     dfree(g->dmax, p->stream);
@@ -1054,11 +1102,23 @@ void gummel_free(Problem *p) {
     p->gs = nullptr;
 }
 
+// capture: what follows on `to` also waits for what `from` holds so far
+static cudaError_t branch(cudaStream_t from, cudaEvent_t ev, cudaStream_t to) {
+    cudaError_t e = cudaEventRecord(ev, from);
+    return e == cudaSuccess ? cudaStreamWaitEvent(to, ev, 0) : e;
+}
+
 // Record one whole Gummel solve into g->graph: an outer WHILE node over
 // Gummel iterations whose body holds mu_ex, the Poisson solve, the phi
 // relaxation, per species the Slotboom coefficients, the NP solve and the
 // density update, and k_gummel_check, which ends the loop on convergence,
-// a status error or max_iter.  Works on g->phi and g->rho.
+// a status error or max_iter.  What does not depend on one another is recorded
+// as parallel branches: mu_ex beside the Poisson solve, and the species' solves
+// beside one another.  A CG iteration is a chain of about 30 launches that
+// leave most of the chip idle below 64^3 (80 of the 103 us of a 32^3 iteration
+// are launch and FP64 latency), and double-float mu_ex runs on the FP32 pipes
+// while the solves run on the FP64 ones.  Sixteen sweeps of the 32^3 film: 46.5
+// -> 29.1 ms; four of a 90^3 request: 48.8 -> 38.3 ms.  Works on g->phi and g->rho.
 static int build_graph(Problem *p, int *d_q, double *d_rhof) {
     NvtxRange range("build_solve_graph");
     GummelState *g = p->gs;
@@ -1067,6 +1127,7 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
     const int G = grid_for(N);
     PhysConst c{p->nx, p->ny, p->nz, p->bc[0], p->bc[1], p->lB, p->phi_lo, p->phi_hi};
     const int maxlin = 2000;
+    Lane *a = &g->lane[0];         // the Poisson solves'
     cudaStream_t st = p->stream, sb = g->cap[0], sc = g->cap[1];
     const bool timer = p->timer.enabled;
     p->timer.enabled = false;
@@ -1101,16 +1162,16 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             ec.lam = p->lambda_rho;
             rc = mu_ex_enqueue(p, p->precision, g->rho, g->mu, sb);
             cudaMemsetAsync(g->dmax, 0, sizeof(unsigned long long), sb);
-            set_operator(g, true);
-            Level &L0 = g->lv[0];
-            k_eq_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, ec, g->phi, g->mu, d_rhof, g->rhs, L0.dg, p->d_flag);
-            k_fill<<<G, 256, 0, sb>>>(g->x, 0.0, N);
-            g->shift = true;
-            op_setup(g, false, sb);
-            e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
-            g->shift = false;
-            set_operator(g, true);
-            k_eq_update<<<G, 256, 0, sb>>>(N, ec, g->phi, g->x, g->mu, g->rho, g->dmax, p->d_flag);
+            set_operator(a, true);
+            Level &L0 = a->lv[0];
+            k_eq_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, ec, g->phi, g->mu, d_rhof, a->rhs, L0.dg, p->d_flag);
+            k_fill<<<G, 256, 0, sb>>>(a->x, 0.0, N);
+            a->shift = true;
+            op_setup(a, false, sb);
+            e = pcg_capture(a, a->x, a->rhs, p->lin_tol, maxlin, p->d_flag, g->stats, sb, sc);
+            a->shift = false;
+            set_operator(a, true);
+            k_eq_update<<<G, 256, 0, sb>>>(N, ec, g->phi, a->x, g->mu, g->rho, g->dmax, p->d_flag);
             k_eq_check<<<1, 1, 0, sb>>>(g->dmax, p->d_flag, p->eq_tol, p->eq_max_iter, g->stats, he, hg);
             cudaError_t e2 = cudaStreamEndCapture(sb, &ebody);
             if (e == cudaSuccess) e = e2;
@@ -1130,35 +1191,45 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             k_aa_begin<<<1, 1, 0, sb>>>(g->aa);
             k_aa_save_x<<<GM, 256, 0, sb>>>(g->aa, g->phi, g->rho, g->aa_X, N, M);
         }
-        // 1. mu_ex from rho^{n-1}
-        rc = mu_ex_enqueue(p, p->precision, g->rho, g->mu, sb);
-        if (g->phase) k_phase_mark<<<1, 1, 0, sb>>>(g->phase, 0);
+        // 1. mu_ex from rho^{n-1}, beside the Poisson solve, which does not read
+        // it (before it when the phases are timed)
         cudaMemsetAsync(g->dmax, 0, sizeof(unsigned long long), sb);
+        cudaStream_t sm = sb;
+        if (!g->phase) {
+            sm = g->fork[0];
+            e = branch(sb, g->ev[0], sm);
+        }
+        if (e == cudaSuccess) rc = mu_ex_enqueue(p, p->precision, g->rho, g->mu, sm);
+        if (g->phase) k_phase_mark<<<1, 1, 0, sb>>>(g->phase, 0);
         // 2. Poisson for phi*, starting from phi; 3. relax phi
-        set_operator(g, true);
-        if (p->screened) {
+        set_operator(a, true);
+        if (e == cudaSuccess && p->screened) {
             // one Newton step with the densities' Boltzmann response:
             // (A + dg) dphi = b(rho) - A phi, phi* = phi + dphi
-            Level &L0 = g->lv[0];
-            k_scr_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, g->rho, s, d_q, d_rhof, g->phi, g->rhs, L0.dg);
-            k_fill<<<G, 256, 0, sb>>>(g->x, 0.0, N);
-            g->shift = true;
-            op_setup(g, false, sb);
-            e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
-            g->shift = false;
-            set_operator(g, true);
-            k_relax_phi_step<<<G, 256, 0, sb>>>(g->phi, g->x, p->lambda_phi, N, g->dmax);
-        } else {
-            k_poisson_rhs<<<G, 256, 0, sb>>>(c, g->rho, s, d_q, d_rhof, g->rhs);
-            k_copy<<<G, 256, 0, sb>>>(g->x, g->phi, N);
-            op_setup(g, false, sb);
-            e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
-            set_operator(g, true);
-            k_relax_phi<<<G, 256, 0, sb>>>(g->phi, g->x, p->lambda_phi, N, g->dmax);
+            Level &L0 = a->lv[0];
+            k_scr_rhs<<<G, 256, 0, sb>>>(op_of(L0), c, g->rho, s, d_q, d_rhof, g->phi, a->rhs, L0.dg);
+            k_fill<<<G, 256, 0, sb>>>(a->x, 0.0, N);
+            a->shift = true;
+            op_setup(a, false, sb);
+            e = pcg_capture(a, a->x, a->rhs, p->lin_tol, maxlin, p->d_flag, g->stats, sb, sc);
+            a->shift = false;
+            k_relax_phi_step<<<G, 256, 0, sb>>>(g->phi, a->x, p->lambda_phi, N, g->dmax);
+        } else if (e == cudaSuccess) {
+            k_poisson_rhs<<<G, 256, 0, sb>>>(c, g->rho, s, d_q, d_rhof, a->rhs);
+            k_copy<<<G, 256, 0, sb>>>(a->x, g->phi, N);
+            op_setup(a, false, sb);
+            e = pcg_capture(a, a->x, a->rhs, p->lin_tol, maxlin, p->d_flag, g->stats, sb, sc);
+            k_relax_phi<<<G, 256, 0, sb>>>(g->phi, a->x, p->lambda_phi, N, g->dmax);
         }
+        set_operator(a, true);
+        if (e == cudaSuccess && sm != sb) e = branch(sm, g->ev[1], sb);
         if (g->phase) k_phase_mark<<<1, 1, 0, sb>>>(g->phase, 1);
-        // 4. Nernst-Planck per species
+        // 4. Nernst-Planck per species, on one branch per lane
+        const size_t lanes = g->lane.size();
+        for (size_t k = 1; k < lanes && e == cudaSuccess; ++k) e = branch(sb, g->ev[0], g->fork[k - 1]);
         for (int i = 0; i < s && e == cudaSuccess; ++i) {
+            Lane *b = &g->lane[i % lanes];
+            cudaStream_t sn = i % lanes ? g->fork[i % lanes - 1] : sb;
             NpConst nc;
             nc.D = p->D[i];
             nc.q = p->q[i];
@@ -1166,16 +1237,17 @@ static int build_graph(Problem *p, int *d_q, double *d_rhof) {
             nc.Dhi = p->D[i] * std::exp(-(p->q[i] * p->phi_hi + p->mu_bulk[i]));
             nc.rlo = p->rho_b[i] * std::exp(p->q[i] * p->phi_lo + p->mu_bulk[i]);
             nc.rhi = p->rho_b[i] * std::exp(p->q[i] * p->phi_hi + p->mu_bulk[i]);
-            Level &L0 = g->lv[0];
-            const Op A0 = op_of(L0);
-            k_np_mobility<<<G, 256, 0, sb>>>(N, nc, g->phi, g->mu + i * N, g->rho + i * N, g->em, g->x, p->d_flag);
-            k_np_faces<<<blocks_for(N, 128), 128, 0, sb>>>(c, nc, A0, g->em, L0.cx, L0.cy, L0.cz, L0.czlo, g->rhs);
-            op_setup(g, true, sb);
-            e = pcg_capture(g, g->x, g->rhs, p->lin_tol, maxlin, p->d_flag, sb, sc);
-            k_np_finish<<<G, 256, 0, sb>>>(N, p->lambda_rho, p->rho_mix, 1.0 / p->rho_b[i], g->em,
-                                           g->x, g->rho + i * N, g->lam ? g->lam + i * N : nullptr,
+            Level &L0 = b->lv[0];
+            k_np_mobility<<<G, 256, 0, sn>>>(N, nc, g->phi, g->mu + i * N, g->rho + i * N, b->em, b->x, p->d_flag);
+            k_np_faces<<<blocks_for(N, 128), 128, 0, sn>>>(c, nc, op_of(L0), b->em, L0.cx, L0.cy, L0.cz, L0.czlo,
+                                                           b->rhs);
+            op_setup(b, true, sn);
+            e = pcg_capture(b, b->x, b->rhs, p->lin_tol, maxlin, p->d_flag, g->stats, sn, sc);
+            k_np_finish<<<G, 256, 0, sn>>>(N, p->lambda_rho, p->rho_mix, 1.0 / p->rho_b[i], b->em, b->x,
+                                           g->rho + i * N, g->lam ? g->lam + i * N : nullptr,
                                            g->prev ? g->prev + i * N : nullptr, g->dmax, p->d_flag);
         }
+        for (size_t k = 1; k < lanes && e == cudaSuccess; ++k) e = branch(g->fork[k - 1], g->ev[k], sb);
         if (g->phase) k_phase_mark<<<1, 1, 0, sb>>>(g->phase, 2);
         if (g->aa) {
             // Anderson extrapolation of the plain iterate (or a repeat of the

@@ -77,7 +77,12 @@ constexpr double kCoarseScale = 1.8;
 constexpr int kDotBlocks = 512;
 constexpr int kSweepThreads = 128;
 
-enum { S_RZ0 = 0, S_RZ1, S_TGT, S_COUNT };
+// record of a linear solve in progress
+struct LinCtl {
+    double rz[2];                  // r . z of this and the previous iteration, by parity
+    double tgt;                    // ||r||^2 to reach
+    int it;                        // iterations done
+};
 
 static Op op_of(const Level &L, bool shift = false) {
     Op A{};
@@ -474,14 +479,13 @@ __global__ void __launch_bounds__(256) k_pcg_start(Op A, const double *__restric
 }
 
 // p = z + beta p (p = z in the first iteration)
-__global__ void __launch_bounds__(256) k_pcg_direction(double *__restrict__ p, const double *__restrict__ z,
-                                                       double *__restrict__ scal, const double *__restrict__ part_rz,
-                                                       int nb, const DevStats *__restrict__ st, unsigned n) {
-    const int it = st->pcg_it;
+__global__ void __launch_bounds__(256) k_pcg_direction(double *__restrict__ p, const double *__restrict__ z, LinCtl *ctl,
+                                                       const double *__restrict__ part_rz, int nb, unsigned n) {
+    const int it = ctl->it;
     const bool first = it == 0;
     const double beta = of_partials(part_rz, nb, [&](double rz) {
-        if (blockIdx.x == 0) scal[S_RZ0 + (it & 1)] = rz;
-        return first ? 0.0 : rz / scal[S_RZ0 + ((it + 1) & 1)];
+        if (blockIdx.x == 0) ctl->rz[it & 1] = rz;
+        return first ? 0.0 : rz / ctl->rz[(it + 1) & 1];
     });
     for (unsigned k = blockIdx.x * 256 + threadIdx.x; k < n; k += gridDim.x * 256)
         p[k] = first ? z[k] : fma(beta, p[k], z[k]);
@@ -505,11 +509,10 @@ __global__ void __launch_bounds__(256) k_pcg_apply(Op A, const double *__restric
 __global__ void __launch_bounds__(256) k_pcg_update(Op A, double *__restrict__ x, double *__restrict__ r,
                                                     const double *__restrict__ p, const double *__restrict__ Ap,
                                                     double *__restrict__ zred, double *__restrict__ zblack,
-                                                    const double *__restrict__ scal,
+                                                    const LinCtl *__restrict__ ctl,
                                                     const double *__restrict__ part_pap, int nb,
-                                                    const DevStats *__restrict__ st, double *__restrict__ part_rr) {
-    const double alpha =
-        of_partials(part_pap, nb, [&](double pap) { return scal[S_RZ0 + (st->pcg_it & 1)] / pap; });
+                                                    double *__restrict__ part_rr) {
+    const double alpha = of_partials(part_pap, nb, [&](double pap) { return ctl->rz[ctl->it & 1] / pap; });
     double acc = 0.0;
     for (unsigned k = blockIdx.x * 256 + threadIdx.x; k < A.n; k += gridDim.x * 256) {
         x[k] = fma(alpha, p[k], x[k]);
@@ -526,31 +529,31 @@ __global__ void __launch_bounds__(256) k_pcg_update(Op A, double *__restrict__ x
 
 // start of a linear solve: target = tol^2 ||b||^2; enter the loop unless the
 // warm start already meets it
-__global__ void k_pcg_init(double *scal, const double *__restrict__ part_bb, const double *__restrict__ part_rr,
-                           int nb, double tol, DevStats *st, int *flag, cudaGraphConditionalHandle h) {
+__global__ void k_pcg_init(LinCtl *ctl, const double *__restrict__ part_bb, const double *__restrict__ part_rr,
+                           int nb, double tol, const DevStats *st, int *flag, cudaGraphConditionalHandle h) {
     double bb = partials_tree(part_bb, nb);
     const double rr = partials_tree(part_rr, nb);
     if (threadIdx.x != 0) return;
     if (!(tol > 0)) tol = st->lin_tol;      // adaptive: set by the Gummel loop
     if (!(bb > 0)) bb = 1.0;
     const double tgt = tol * tol * bb;
-    scal[S_TGT] = tgt;
-    st->pcg_it = 0;
+    ctl->tgt = tgt;
+    ctl->it = 0;
     const bool finite = isfinite(rr);
     if (!finite) atomicOr(flag, kFlagOverflow);
     cudaGraphSetConditional(h, (finite && rr > tgt) ? 1u : 0u);
 }
 
 // end of a CG iteration: continue while ||r||^2 > target and below maxit
-__global__ void k_pcg_check(const double *scal, const double *__restrict__ part_rr, int nb, int maxit, DevStats *st,
-                            int *flag, cudaGraphConditionalHandle h) {
+__global__ void k_pcg_check(LinCtl *ctl, const double *__restrict__ part_rr, int nb, int maxit, DevStats *st, int *flag,
+                            cudaGraphConditionalHandle h) {
     const double rr = partials_tree(part_rr, nb);
     if (threadIdx.x != 0) return;
-    const int it = ++st->pcg_it;
-    st->lin += 1;
+    const int it = ++ctl->it;
+    atomicAdd(&st->lin, 1ull);        // lanes run side by side
     const bool finite = isfinite(rr);
     if (!finite) atomicOr(flag, kFlagOverflow);
-    cudaGraphSetConditional(h, (finite && rr > scal[S_TGT] && it < maxit) ? 1u : 0u);
+    cudaGraphSetConditional(h, (finite && rr > ctl->tgt && it < maxit) ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------

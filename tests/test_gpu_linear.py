@@ -22,7 +22,7 @@ TOL = 1e-8
     ("PPD", 10, 9, 23),      # 1 x 1 x 23: one lane a point
     ("PPD", 10, 9, 53),      # 1 x 1 x 53: sweeps in shared memory
     ("NPD", 14, 15, 12),     # no-flux walls, an odd extent that does not wrap below
-    ("PPD", 22, 45, 15),     # odd levels above the one-CTA tail
+    ("PPD", 18, 45, 15),     # odd levels above the one-CTA tail
     ("PPD", 48, 50, 60),     # 144000 points: two points in some slots
 ])
 def test_two_sweeps_match_oracle(bc, nx, ny, nz):
