@@ -855,6 +855,37 @@ static bool launch_zreg(bool back, int s, bool msa, typename vec2<T>::type *B10,
     }
 }
 
+// z kernels in the wide form where the paired-column form's warps would not
+// give every quarter of an SM one (kWideWarps); false otherwise.  The MSA term
+// stays with the paired-column kernel.
+constexpr long kWideWarps = 4 * 152;
+template <typename T, int N1, int N2>
+static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>::type *B10,
+                         typename vec2<T>::type *Bs, const Dims &d, const typename vec2<T>::type *twz, const T *spec,
+                         const SpeciesConst &sc, cudaStream_t st) {
+    if constexpr (N1 * N2 > kWideMaxLen) {
+        return false;
+    } else {
+        constexpr int G = Shape<N1, N2>::G;
+        if (plain_warps >= kWideWarps || (back && msa) || sc.s > kWideGroups) return false;
+        int TX = 1;
+        while (TX < 4 && 4 * TX * G * kWideGroups <= kWideThreads &&
+               wide_smem<T, N1, N2>(back, sc.s, 2 * TX) <= (size_t)96 * 1024)
+            TX *= 2;
+        const size_t sm = wide_smem<T, N1, N2>(back, sc.s, TX);
+        if (2 * TX * G * kWideGroups > kWideThreads || sm > (size_t)kSmemCap) return false;
+        const dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
+        if (back) {
+            ensure_smem<k_zback_w<T, N1, N2>>();
+            k_zback_w<T, N1, N2><<<g, 2 * TX * G * kWideGroups, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);
+        } else {
+            ensure_smem<k_zmac_w<T, N1, N2>>();
+            k_zmac_w<T, N1, N2><<<g, 2 * TX * G * kWideGroups, sm, st>>>(Bs, B10, d, twz, spec, sc, TX);
+        }
+        return true;
+    }
+}
+
 template <typename T>
 static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, double *d_mu, cudaStream_t st,
                         bool tc = false) {
@@ -944,14 +975,20 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
                 constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
                 if (launch_zreg<T, N1, N2>(back, s, sc.msa != 0, B10, Bs, d, twz, spec, sc, st)) return;
                 // paired columns (ky, Ly - ky): 2 TX columns per CTA
-                const long per_col = ((long)s * N1 * G + Shape<N1, N2>::EX) * (long)cs;
+                // a lane t < N2 keeps N1 values per species and column: N1 N2
+                // slots (with N1 lanes' worth of them, L = 80 ran 8 warps per SM)
+                const long per_col = ((long)s * N1 * N2 + Shape<N1, N2>::EX) * (long)cs;
                 int TX = pow2_le(std::max<long>(1, std::min<long>(std::min<long>(128 / G, 8), kBudget / (2 * per_col))));
+                while (TX > 1 && (long)((d.Wx + TX - 1) / TX) * (d.Ly / 2 + 1) < 2 * 152) TX /= 2;
                 if (p->tile[2] > 0)
                     TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
                                                                                     (kSmemCap - (long)G * G * cs) /
                                                                                         (2 * per_col))));
                 dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
                 const size_t sm = 2 * TX * per_col + (size_t)G * G * cs;   // + twiddle table
+                if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)g.x * g.y * ((2 * TX * G + 31) / 32), B10, Bs, d, twz,
+                                            spec, sc, st))
+                    return;
                 if (back && sc.msa) {
                     ensure_smem<k_zback_p<T, N1, N2, true>>();
                     k_zback_p<T, N1, N2, true><<<g, 2 * TX * G, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);

@@ -366,17 +366,17 @@ __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__
     const int c = threadIdx.x % TX, b = (threadIdx.x / TX) & 1, t = threadIdx.x / (2 * TX);
     const int lanes = 2 * TX;                        // interleaved columns in the tile
     const int col = b * TX + c;
-    C *slots = reinterpret_cast<C *>(smem_raw);      // [s][N1][G][2 TX]
-    C *ex = slots + (size_t)sc.s * N1 * G * lanes + col;
-    const int rstride = N1 * G * lanes;
-    auto slot = [&](int i, int k1) -> C & { return slots[i * rstride + (k1 * G + t) * lanes + col]; };
+    C *slots = reinterpret_cast<C *>(smem_raw);      // [s][N1][N2][2 TX]
+    C *ex = slots + (size_t)sc.s * N1 * N2 * lanes + col;
+    const int rstride = N1 * N2 * lanes;
+    auto slot = [&](int i, int k1) -> C & { return slots[i * rstride + (k1 * N2 + t) * lanes + col]; };
     const int kyp = blockIdx.y, kx = blockIdx.x * TX + c;
     int ky;
     const bool ok = zcol(d, kyp, b, kx, ky);
     const size_t plane = (size_t)d.Ly * d.Wx;
     // 64-bit types: lane twiddles from a shared table (frees 2 G registers);
     // FP32 keeps them in registers
-    C *twtab = slots + (size_t)sc.s * N1 * G * lanes + (size_t)Shape<N1, N2>::EX * lanes;
+    C *twtab = slots + (size_t)sc.s * N1 * N2 * lanes + (size_t)Shape<N1, N2>::EX * lanes;
     using TwT = typename std::conditional<std::is_same<T, float>::value, LaneTw<N1, N2, C>, SmemTw<N1, N2, C>>::type;
     TwT lt;
     if constexpr (std::is_same<T, float>::value) {
@@ -460,17 +460,17 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
     const int c = threadIdx.x % TX, b = (threadIdx.x / TX) & 1, t = threadIdx.x / (2 * TX);
     const int lanes = 2 * TX;
     const int col = b * TX + c;
-    C *slots = reinterpret_cast<C *>(smem_raw);      // accumulators [s][N1][G][2 TX]
-    C *ex = slots + (size_t)sc.s * N1 * G * lanes + col;
-    const int rstride = N1 * G * lanes;
-    auto slot = [&](int i, int k1) -> C & { return slots[i * rstride + (k1 * G + t) * lanes + col]; };
+    C *slots = reinterpret_cast<C *>(smem_raw);      // accumulators [s][N1][N2][2 TX]
+    C *ex = slots + (size_t)sc.s * N1 * N2 * lanes + col;
+    const int rstride = N1 * N2 * lanes;
+    auto slot = [&](int i, int k1) -> C & { return slots[i * rstride + (k1 * N2 + t) * lanes + col]; };
     const int kyp = blockIdx.y, kx = blockIdx.x * TX + c;
     int ky;
     const bool ok = zcol(d, kyp, b, kx, ky);
     const size_t plane = (size_t)d.Ly * d.Wx;
     // 64-bit types: lane twiddles from a shared table (frees 2 G registers);
     // FP32 keeps them in registers
-    C *twtab = slots + (size_t)sc.s * N1 * G * lanes + (size_t)Shape<N1, N2>::EX * lanes;
+    C *twtab = slots + (size_t)sc.s * N1 * N2 * lanes + (size_t)Shape<N1, N2>::EX * lanes;
     using TwT = typename std::conditional<std::is_same<T, float>::value, LaneTw<N1, N2, C>, SmemTw<N1, N2, C>>::type;
     TwT lt;
     if constexpr (std::is_same<T, float>::value) {
@@ -573,6 +573,209 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
                 const int zz = t + N1 * n2;
                 if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
             }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// z kernels, wide form, for grids whose column tiles do not fill the chip.  In
+// the paired-column kernels above a warp runs all transforms of its columns in
+// turn: s + 10 of them and the products, a chain that a 20^3 grid spreads over
+// 66 warps for 608 quarter-SMs, each FP64 instruction holding its quarter for 64
+// clocks.  Here ten thread groups share a column tile: a transform runs in a
+// group of its own, the spectra meet in shared memory, and the chain is one
+// transform, one group's products and one transform.  Same operations in the
+// same order.  z MAC / z back, us: 16^3 FP64 84 / 85 -> 30 / 24, 32^3 FP64 97 / 100
+// -> 59 / 46, double-float 62 / 55 -> 26 / 22, 48^3 double-float 70 / 64 -> 39 / 31.
+constexpr int kWideGroups = kNumWeighted;
+constexpr int kWideThreads = 512;
+constexpr int kWideMaxLen = 96;       // longer columns come in grids that fill the chip
+
+// kernel type and weighted density of entry `e` of the order in which the
+// products are summed: shell {n0, n1, n2}, ball {n3}, vector x {n1x, n2x}, y, z
+__device__ __forceinline__ void wide_entry(int e, int &type, int &alpha) {
+    type = e < 3 ? 0 : (e < 4 ? 1 : 2 + (e - 4) / 2);
+    alpha = e < 4 ? e : ((e & 1) ? 7 + type - 2 : 4 + type - 2);
+}
+
+template <typename T> __device__ __forceinline__ T wide_factor(const SpeciesConst &sc, int alpha, int i) {
+    return alpha == 0 ? sc_c0<T>(sc, i) : ((alpha == 1 || (alpha >= 4 && alpha < 7)) ? sc_c1<T>(sc, i) : (T)1);
+}
+
+template <typename T, int N1, int N2> static size_t wide_smem(bool back, int s, int TX) {
+    constexpr size_t G = Shape<N1, N2>::G;
+    const size_t spectra = (size_t)((back ? kWideGroups : 0) + s) * N1 * N2;
+    return (2 * TX * (spectra + (size_t)kWideGroups * Shape<N1, N2>::EX) + G * G) * sizeof(typename vec2<T>::type);
+}
+
+// place of a thread: group, lane t, column (b, c) of the tile
+struct WideLane {
+    int grp, t, col, lanes, ky, kx;
+    bool ok;
+    __device__ __forceinline__ WideLane(const Dims &d, int TX, int G) {
+        const int c = threadIdx.x % TX, b = (threadIdx.x / TX) & 1;
+        t = (threadIdx.x / (2 * TX)) % G;
+        grp = threadIdx.x / (2 * TX * G);
+        lanes = 2 * TX;
+        col = b * TX + c;
+        kx = blockIdx.x * TX + c;
+        ok = zcol(d, blockIdx.y, b, kx, ky);
+    }
+};
+
+template <typename T, int N1, int N2>
+__global__ void __launch_bounds__(kWideThreads) k_zmac_w(const typename vec2<T>::type *__restrict__ Bs,
+                                                         typename vec2<T>::type *__restrict__ B10, Dims d,
+                                                         const typename vec2<T>::type *__restrict__ tw,
+                                                         const T *__restrict__ spec, SpeciesConst sc, int TX) {
+    using C = typename vec2<T>::type;
+    constexpr int G = Shape<N1, N2>::G, EX = Shape<N1, N2>::EX;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const WideLane w(d, TX, G);
+    const int t = w.t, lanes = w.lanes;
+    C *rho = reinterpret_cast<C *>(smem_raw);        // [s][N1][N2][2 TX]
+    C *ex0 = rho + (size_t)sc.s * N1 * N2 * lanes;    // [group][EX][2 TX]
+    C *twtab = ex0 + (size_t)kWideGroups * EX * lanes;
+    C *ex = ex0 + (size_t)w.grp * EX * lanes + w.col;
+    SmemTw<N1, N2, C>::fill(twtab, tw);
+    __syncthreads();
+    SmemTw<N1, N2, C> lt;
+    lt.tab = twtab;
+    lt.t = t;
+    const size_t plane = (size_t)d.Ly * d.Wx;
+    C v[G];
+    if (t < N1) {
+        const C *src = Bs + (size_t)w.grp * d.nz * plane + (size_t)w.ky * d.Wx + w.kx;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+            const int zz = t + N1 * n2;
+            v[n2] = (w.ok && w.grp < sc.s && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
+        }
+    }
+    // groups beyond the species have no line: a lane past both factors only
+    // keeps the barriers
+    fwd2<N1, N2>(v, lt, ex, w.grp < sc.s ? t : N1 + N2, lanes);
+    if (t < N2 && w.grp < sc.s) {
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) rho[((w.grp * N1 + k1) * N2 + t) * lanes + w.col] = v[k1];
+    }
+    __syncthreads();
+    int type, alpha;
+    wide_entry(w.grp, type, alpha);
+    if (t < N2) {
+        T g[kChunk][N1];
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) v[k1] = C{0, 0};
+        for (int i0 = 0; i0 < sc.s; i0 += kChunk) {
+            load_spec<T, N1, N2>(g, spec, d, sc.s, i0, type, w.kx, w.ky, t, w.ok);
+#pragma unroll
+            for (int j = 0; j < kChunk; ++j) {
+                const int i = i0 + j;
+                if (i >= sc.s) break;
+                const T cf = wide_factor<T>(sc, alpha, i);
+#pragma unroll
+                for (int k1 = 0; k1 < N1; ++k1) {
+                    const T gg = cf * g[j][k1];
+                    const C x = rho[((i * N1 + k1) * N2 + t) * lanes + w.col];
+                    if (type <= 1) {
+                        v[k1].x += gg * x.x;
+                        v[k1].y += gg * x.y;
+                    } else {             // conj(K) = +i S
+                        v[k1].x -= gg * x.y;
+                        v[k1].y += gg * x.x;
+                    }
+                }
+            }
+        }
+    }
+    inv2<N1, N2>(v, lt, ex, t, lanes);
+    if (t < N1 && w.ok) {
+        C *dst = B10 + (size_t)alpha * d.nz * plane + (size_t)w.ky * d.Wx + w.kx;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+            const int zz = t + N1 * n2;
+            if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
+        }
+    }
+}
+
+template <typename T, int N1, int N2>
+__global__ void __launch_bounds__(kWideThreads) k_zback_w(const typename vec2<T>::type *__restrict__ B10,
+                                                          typename vec2<T>::type *__restrict__ Bs, Dims d,
+                                                          const typename vec2<T>::type *__restrict__ tw,
+                                                          const T *__restrict__ spec, SpeciesConst sc, int TX) {
+    using C = typename vec2<T>::type;
+    constexpr int G = Shape<N1, N2>::G, EX = Shape<N1, N2>::EX;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const WideLane w(d, TX, G);
+    const int t = w.t, lanes = w.lanes;
+    C *psi = reinterpret_cast<C *>(smem_raw);                       // [group][N1][N2][2 TX]
+    C *mu = psi + (size_t)kWideGroups * N1 * N2 * lanes;            // [s][N1][N2][2 TX]
+    C *ex0 = mu + (size_t)sc.s * N1 * N2 * lanes;
+    C *twtab = ex0 + (size_t)kWideGroups * EX * lanes;
+    C *ex = ex0 + (size_t)w.grp * EX * lanes + w.col;
+    auto place = [&](int a, int k1) { return ((a * N1 + k1) * N2 + t) * lanes + w.col; };
+    SmemTw<N1, N2, C>::fill(twtab, tw);
+    __syncthreads();
+    SmemTw<N1, N2, C> lt;
+    lt.tab = twtab;
+    lt.t = t;
+    const size_t plane = (size_t)d.Ly * d.Wx;
+    C v[G];
+    if (t < N1) {
+        int type, alpha;
+        wide_entry(w.grp, type, alpha);
+        const C *src = B10 + (size_t)alpha * d.nz * plane + (size_t)w.ky * d.Wx + w.kx;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+            const int zz = t + N1 * n2;
+            v[n2] = (w.ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
+        }
+    }
+    fwd2<N1, N2>(v, lt, ex, t, lanes);
+    if (t < N2) {
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) psi[place(w.grp, k1)] = v[k1];
+    }
+    __syncthreads();
+    if (t < N2) {
+        const int fy = w.ky <= d.Ly / 2 ? w.ky : d.Ly - w.ky;
+        const size_t oct = (size_t)d.Ox * d.Oy * d.Oz;
+        for (int e = w.grp; e < sc.s * N1; e += kWideGroups) {
+            const int i = e / N1, k1 = e - i * N1, kz = t + N2 * k1, fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
+            const T *base = spec + (size_t)i * kNumKernels * oct + ((size_t)fz * d.Oy + fy) * d.Ox + w.kx;
+            C acc = C{0, 0};
+#pragma unroll
+            for (int q = 0; q < kWideGroups; ++q) {
+                int type, alpha;
+                wide_entry(q, type, alpha);
+                T g = w.ok ? ldgt(&base[type * oct]) : (T)0;
+                if ((type == 3 && w.ky > d.Ly / 2) || (type == 4 && kz > d.Lz / 2)) g = -g;
+                const T gg = wide_factor<T>(sc, alpha, i) * g;
+                const C x = psi[place(q, k1)];
+                if (type <= 1) {
+                    acc.x += gg * x.x;
+                    acc.y += gg * x.y;
+                } else {             // K = -i S
+                    acc.x += gg * x.y;
+                    acc.y -= gg * x.x;
+                }
+            }
+            mu[place(i, k1)] = acc;
+        }
+    }
+    __syncthreads();
+    if (t < N2 && w.grp < sc.s) {
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) v[k1] = mu[place(w.grp, k1)];
+    }
+    inv2<N1, N2>(v, lt, ex, w.grp < sc.s ? t : N1 + N2, lanes);
+    if (t < N1 && w.ok && w.grp < sc.s) {
+        C *dst = Bs + (size_t)w.grp * d.nz * plane + (size_t)w.ky * d.Wx + w.kx;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+            const int zz = t + N1 * n2;
+            if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
         }
     }
 }
