@@ -97,6 +97,14 @@ bool host_values_ok(const double *x, size_t n, int kind) {
     return true;
 }
 
+// One byte per page is read and written back: a page of fresh memory faulted in
+// here costs a fraction of one that the copy from the device faults in.
+void touch_pages(void *x, size_t bytes) {
+    volatile char *c = (volatile char *)x;
+    for (size_t k = 0; k < bytes; k += 4096) c[k] = c[k];
+    if (bytes) c[bytes - 1] = c[bytes - 1];
+}
+
 void dfree(void *ptr, cudaStream_t st) {
     if (ptr) cudaFreeAsync(ptr, st);
 }
@@ -156,6 +164,7 @@ static int read_flag(Problem *p, cudaStream_t st) {
         cudaMemsetAsync(p->d_flag, 0, sizeof(int), st);
         cudaStreamSynchronize(st);
     }
+    if (h & kFlagInvalid) return PNP_ERR_INVALID;
     if (h & kFlagTimeout) return PNP_ERR_TIMEOUT;
     if (h & kFlagOverflow) return PNP_ERR_OVERFLOW;
     if (h & (kFlagPacking | kFlagNonFinite)) return PNP_ERR_PACKING;
@@ -326,7 +335,6 @@ int pnp_excess_mu(pnp_problem *h, const double *rho, double *mu_ex, int precisio
     int prec = resolve_prec(p, precision);
     if (prec < 0) return PNP_ERR_INVALID;
     const size_t n = p->npts() * p->s;
-    if (!host_values_ok(rho, n, 1)) return PNP_ERR_INVALID;
     if (!p->d_io) {
         if (dmalloc((void **)&p->d_io, sizeof(double) * (2 * n + p->npts()), p->stream) != cudaSuccess)
             return PNP_ERR_NOMEM;
@@ -334,14 +342,22 @@ int pnp_excess_mu(pnp_problem *h, const double *rho, double *mu_ex, int precisio
     }
     cudaStream_t st = p->stream;
     p->last_stream = st;
+    // The densities are checked on the device, and the pages of a fresh output
+    // array are touched while it computes: the host's scan and the page faults
+    // of the copy back were 0.55 and 0.40 of the 0.86 ms of a 64^3 FP32 call.
+    // Nothing is copied back for densities that fail the check.
     cudaError_t e = cudaMemcpyAsync(p->d_io, rho, sizeof(double) * n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->d_flag, 0, sizeof(int), st);
     if (e != cudaSuccess) return cuda_status(e);
-    int rc = mu_ex_enqueue(p, prec, p->d_io, p->d_io + n, st);
+    int rc = check_values_enqueue(p, p->d_io, n, st);
+    if (rc == PNP_OK) rc = mu_ex_enqueue(p, prec, p->d_io, p->d_io + n, st);
     if (rc) return rc;
+    touch_pages(mu_ex, sizeof(double) * n);
+    rc = read_flag(p, st);
+    if (rc != PNP_OK && rc != PNP_ERR_PACKING && rc != PNP_ERR_OVERFLOW && rc != PNP_ERR_TIMEOUT) return rc;
     e = cudaMemcpyAsync(mu_ex, p->d_io + n, sizeof(double) * n, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return cuda_status(e);
-    return read_flag(p, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? rc : cuda_status(e);
 }
 
 int pnp_excess_mu_device(pnp_problem *h, const double *d_rho, double *d_mu_ex, int precision, void *stream) {
@@ -399,7 +415,12 @@ int pnp_gummel_solve(pnp_problem *h, const double *phi0, const double *rho0, dou
     }
     if (e != cudaSuccess) return fail(cuda_status(e));
     pnp_stats local{};
-    int rc = gummel_run(p, d_phi0, d_rho0, d_phi, d_rho, &local, st);
+    // the output's pages are touched while the device solves (as in pnp_excess_mu:
+    // the copy back into 134 MB of fresh memory takes 5.8 ms, into touched 0.7)
+    int rc = gummel_run(p, d_phi0, d_rho0, d_phi, d_rho, &local, st, [&] {
+        if (phi_out) touch_pages(phi_out, sizeof(double) * N);
+        if (rho_out) touch_pages(rho_out, sizeof(double) * n);
+    });
     if (rc == PNP_OK || rc == PNP_ERR_NOT_CONVERGED) {
         if (phi_out) e = cudaMemcpyAsync(phi_out, d_phi, sizeof(double) * N, cudaMemcpyDeviceToHost, st);
         if (rho_out && e == cudaSuccess)

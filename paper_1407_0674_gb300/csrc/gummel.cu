@@ -1388,9 +1388,10 @@ void gummel_decode_stats(const void *raw, pnp_stats *out) {
 }
 
 int gummel_run(Problem *p, const double *d_phi0, const double *d_rho0, double *d_phi, double *d_rho, pnp_stats *stats,
-               cudaStream_t st) {
+               cudaStream_t st, const std::function<void()> &meanwhile) {
     int rc = gummel_launch(p, d_phi0, d_rho0, st);
     if (rc) return rc;
+    if (meanwhile) meanwhile();
     DevStats hs;
     rc = gummel_fetch(p, d_phi, d_rho, &hs, st);
     if (rc) return rc;

@@ -436,6 +436,20 @@ int mu_ex_enqueue(Problem *p, int prec, const double *d_rho, double *d_mu, cudaS
     return run_pipeline_fp32(p, p->buf[1], d_rho, d_mu, st, prec == PNP_PREC_TF32SPLIT);
 }
 
+// The check of a host call's densities, on the device copy: the host's scan of
+// 64^3 x 3 values took 0.55 ms of a 0.86 ms call, this 3 us.
+static __global__ void k_check_values(const double *__restrict__ x, size_t n, int *__restrict__ flag) {
+    bool ok = true;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        ok = ok && x[i] >= 0.0 && isfinite(x[i]);
+    if (!ok) atomicOr(flag, kFlagInvalid);
+}
+
+int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st) {
+    k_check_values<<<(int)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(d, n, p->d_flag);
+    return cuda_status(cudaGetLastError());
+}
+
 // ---------------------------------------------------------------------------
 // stage timing
 cudaEvent_t StageTimer::get() {

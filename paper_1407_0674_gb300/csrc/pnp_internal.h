@@ -6,6 +6,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -154,13 +155,16 @@ int mu_ex_setup(Problem *p);                 // workspace, spectra, mu_sh
 int mu_ex_prepare(Problem *p, int prec);     // lazily build one precision's buffers
 int mu_ex_enqueue(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st);
 void mu_ex_free(Problem *p);
+// sets kFlagInvalid in p->d_flag unless every d[k] is finite and >= 0
+int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st);
 // F_sh (Sec 2.3.2) of device densities into d_out[0] (d_part: 512 doubles)
 int square_well_energy_enqueue(Problem *p, const double *d_rho, double *d_out, double *d_part, cudaStream_t st);
 
 // gummel.cu
 int gummel_setup(Problem *p);
+// `meanwhile`: host work done while the device solves
 int gummel_run(Problem *p, const double *d_phi0, const double *d_rho0, double *d_phi, double *d_rho,
-               pnp_stats *stats, cudaStream_t st);
+               pnp_stats *stats, cudaStream_t st, const std::function<void()> &meanwhile = nullptr);
 void gummel_free(Problem *p);
 int plane_flux(Problem *p, int species, const double *d_phi, const double *d_mu, const double *d_rho,
                double *d_flux, cudaStream_t st);
@@ -179,12 +183,14 @@ int cuda_status(cudaError_t e);
 cudaError_t dmalloc(void **ptr, size_t bytes, cudaStream_t st);
 // caller arrays: kind 0 finite, 1 >= 0 and finite, 2 > 0 and finite
 bool host_values_ok(const double *x, size_t n, int kind);
+// touches every page of a caller's output array, leaving its contents
+void touch_pages(void *x, size_t bytes);
 void dfree(void *ptr, cudaStream_t st);
 int create_problem_internal(const pnp_problem_desc *desc, Problem **out, std::string *why);
 void destroy_problem_internal(Problem *p);
 
 // device status bits
-enum : int { kFlagPacking = 1, kFlagOverflow = 2, kFlagNonFinite = 4, kFlagTimeout = 8 };
+enum : int { kFlagPacking = 1, kFlagOverflow = 2, kFlagNonFinite = 4, kFlagTimeout = 8, kFlagInvalid = 16 };
 
 }  // namespace pnp
 
