@@ -350,7 +350,7 @@ int pnp_excess_mu(pnp_problem *h, const double *rho, double *mu_ex, int precisio
     if (e == cudaSuccess) e = cudaMemsetAsync(p->d_flag, 0, sizeof(int), st);
     if (e != cudaSuccess) return cuda_status(e);
     int rc = check_values_enqueue(p, p->d_io, n, st);
-    if (rc == PNP_OK) rc = mu_ex_enqueue(p, prec, p->d_io, p->d_io + n, st);
+    if (rc == PNP_OK) rc = mu_ex_launch(p, prec, p->d_io, p->d_io + n, st);
     if (rc) return rc;
     touch_pages(mu_ex, sizeof(double) * n);
     rc = read_flag(p, st);
@@ -367,7 +367,7 @@ int pnp_excess_mu_device(pnp_problem *h, const double *d_rho, double *d_mu_ex, i
     if (prec < 0) return PNP_ERR_INVALID;
     cudaStream_t st = stream ? (cudaStream_t)stream : p->stream;
     p->last_stream = st;
-    return mu_ex_enqueue(p, prec, d_rho, d_mu_ex, st);
+    return mu_ex_launch(p, prec, d_rho, d_mu_ex, st);
 }
 
 int pnp_status(pnp_problem *h) {

@@ -451,6 +451,96 @@ int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------
+// One mu_ex call as a graph, for grids whose kernels are shorter than their
+// launches: eleven launches cost the host 66 us, so a 16^3 FP64 call among others
+// took 67 us; as one graph launch with its two pointer arguments set anew it
+// takes 34, what its kernels take on three streams.  Larger grids hide the
+// launches behind the kernels (kGraphPoints: about 80 us of FP32 kernels).  Recorded on a
+// problem's third call of a precision, so that a program of one or two calls
+// does not pay the recording; the workspace, tables and tiles the other nodes
+// point to belong to the problem and do not change.
+constexpr size_t kGraphPoints = 400000;       // species x grid points
+constexpr int kGraphAfter = 2;
+struct MuGraph {
+    int calls = 0;
+    bool failed = false;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaGraphNode_t node[2] = {nullptr, nullptr};       // first (reads rho) and last (writes mu_ex)
+    cudaKernelNodeParams prm[2] = {};
+    std::vector<void *> args[2];                        // their arguments; the pointer's place is below
+};
+static const int kPointerArg[2] = {0, 1};               // x forward: (in, ...); x inverse: (A, out, ...)
+
+static void free_mu_graph(MuGraph *m) {
+    if (!m) return;
+    if (m->exec) cudaGraphExecDestroy(m->exec);
+    if (m->graph) cudaGraphDestroy(m->graph);
+    delete m;
+}
+
+static bool record_mu_graph(Problem *p, int prec, const double *d_rho, double *d_mu, MuGraph *m) {
+    cudaStream_t cap = nullptr;
+    if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return false;
+    bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed) == cudaSuccess;
+    if (ok) {
+        ok = mu_ex_enqueue(p, prec, d_rho, d_mu, cap) == PNP_OK;
+        ok = cudaStreamEndCapture(cap, &m->graph) == cudaSuccess && ok;
+    }
+    cudaStreamDestroy(cap);
+    // a chain of kernels: one root, one node without dependents
+    size_t n = 0, roots = 1;
+    if (ok) ok = cudaGraphGetNodes(m->graph, nullptr, &n) == cudaSuccess && n > 1;
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (ok) ok = cudaGraphGetNodes(m->graph, nodes.data(), &n) == cudaSuccess;
+    if (ok) ok = cudaGraphGetRootNodes(m->graph, &m->node[0], &roots) == cudaSuccess && roots == 1;
+    for (size_t k = 0; ok && k < n; ++k) {
+        size_t deps = 0;
+        ok = cudaGraphNodeGetDependentNodes(nodes[k], nullptr, nullptr, &deps) == cudaSuccess;
+        if (ok && deps == 0) m->node[1] = nodes[k];
+    }
+    const bool reg = with_shape(p->L[0], [](auto, auto) {});
+    const int count[2] = {reg ? 6 : 7, reg ? 9 : 10};   // arguments of k_xfwd_r or k_xfwd, k_xinv_r or k_xinv
+    for (int k = 0; ok && k < 2; ++k) {
+        ok = m->node[k] && cudaGraphKernelNodeGetParams(m->node[k], &m->prm[k]) == cudaSuccess;
+        if (ok) m->args[k].assign(m->prm[k].kernelParams, m->prm[k].kernelParams + count[k]);
+    }
+    return ok && cudaGraphInstantiate(&m->exec, m->graph, 0) == cudaSuccess;
+}
+
+// One call's mu_ex on `st`: the recorded graph where the problem has one,
+// launches otherwise (large grids, first calls, stage timing, a stream that is
+// being captured).
+int mu_ex_launch(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st) {
+    if (p->npts() * p->s > kGraphPoints || p->timer.enabled) return mu_ex_enqueue(p, prec, d_rho, d_mu, st);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t q = cudaStreamIsCapturing(st, &cs);
+    if (q != cudaSuccess) cudaGetLastError();
+    if (q != cudaSuccess || cs != cudaStreamCaptureStatusNone) return mu_ex_enqueue(p, prec, d_rho, d_mu, st);
+    MuGraph *&m = p->mug[prec];
+    if (!m) m = new MuGraph();
+    if (m->failed || m->calls < kGraphAfter) {
+        m->calls++;
+        return mu_ex_enqueue(p, prec, d_rho, d_mu, st);
+    }
+    if (!m->exec && !record_mu_graph(p, prec, d_rho, d_mu, m)) {
+        cudaGetLastError();
+        m->failed = true;
+        return mu_ex_enqueue(p, prec, d_rho, d_mu, st);
+    }
+    NvtxRange range("mu_ex");
+    const void *ptr[2] = {d_rho, d_mu};
+    for (int k = 0; k < 2; ++k) {
+        cudaKernelNodeParams prm = m->prm[k];
+        m->args[k][kPointerArg[k]] = &ptr[k];
+        prm.kernelParams = m->args[k].data();
+        const cudaError_t e = cudaGraphExecKernelNodeSetParams(m->exec, m->node[k], &prm);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    return cuda_status(cudaGraphLaunch(m->exec, st));
+}
+
+// ---------------------------------------------------------------------------
 // stage timing
 cudaEvent_t StageTimer::get() {
     if (!pool.empty()) {
@@ -521,6 +611,10 @@ void StageTimer::release() {
 
 void mu_ex_free(Problem *p) {
     p->timer.release();
+    for (MuGraph *&m : p->mug) {
+        free_mu_graph(m);
+        m = nullptr;
+    }
     for (int k = 0; k < 3; ++k) {
         free_buffers(p->buf[k], p->stream);
         p->buf[k] = nullptr;

@@ -62,6 +62,7 @@ struct StageTimer {
     void release();
 };
 struct GummelState;     // device state of the Gummel solve
+struct MuGraph;         // one mu_ex call recorded as a graph (mu_ex.cu)
 
 struct Problem {
     // ---- descriptor (copied) ----
@@ -116,6 +117,7 @@ struct Problem {
     size_t device_bytes = 0;
     int deferred = 0;                 // host-side deferred status
     StageTimer timer;
+    MuGraph *mug[4] = {nullptr, nullptr, nullptr, nullptr};   // small grids: one call as a graph, per precision
     int mg_levels = 0;
     int tile[3] = {0, 0, 0};          // register-FFT CTA tiles (x lines, y columns, z columns); 0: rule
     double tuned_ms = 0;              // mu_ex time measured by the autotuner
@@ -154,6 +156,7 @@ int autotune_create(const pnp_problem_desc *desc, Problem **out, std::string *wh
 int mu_ex_setup(Problem *p);                 // workspace, spectra, mu_sh
 int mu_ex_prepare(Problem *p, int prec);     // lazily build one precision's buffers
 int mu_ex_enqueue(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st);
+int mu_ex_launch(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st);   // one call's work
 void mu_ex_free(Problem *p);
 // sets kFlagInvalid in p->d_flag unless every d[k] is finite and >= 0
 int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st);

@@ -1,0 +1,90 @@
+"""mu_ex calls: the recorded graph of small grids against the launches it
+replaces, and the checks of host calls.
+
+Both forms run the same kernels on the same values, so results are equal bit
+for bit; wide z kernels are compared with the oracle at the parity bar (1e-10).
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from workloads import mu_microbench
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pnp():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1407_0674_gb300 import build, pnp as mod
+    build.build()
+    return mod
+
+
+@pytest.mark.parametrize("precision", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("shape", [(12, 12, 12), (33, 9, 14)])
+def test_graph_calls_equal_launches(pnp, precision, shape):
+    import torch
+    spec, rho = mu_microbench(shape=shape)
+    ins = [torch.from_numpy(rho * f).cuda() for f in (1.0, 0.5, 0.9)]
+    with pnp.Problem(spec, precision=precision) as P:
+        want = []
+        P.stage_timing(True)                  # timed calls are launched one by one
+        for d in ins:
+            out = torch.empty_like(d)
+            P.excess_mu_device(d, out)
+            assert P.status() == pnp.OK
+            want.append(out.cpu().numpy())
+        P.stage_timing(False)
+        side = torch.cuda.Stream()
+        for k in range(9):                    # fresh buffers, two streams
+            d, out = ins[k % 3].clone(), torch.full_like(ins[0], np.nan)
+            torch.cuda.synchronize()
+            P.excess_mu_device(d, out, stream=side.cuda_stream if k % 2 else None)
+            assert P.status() == pnp.OK
+            assert np.array_equal(out.cpu().numpy(), want[k % 3])
+        # a stream under capture records the launches
+        d, out = ins[1].clone(), torch.zeros_like(ins[0])
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            P.excess_mu_device(d, out, stream=torch.cuda.current_stream().cuda_stream)
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want[1])
+
+
+def test_host_call_checks_values(pnp):
+    spec, rho = mu_microbench(10)
+    with pnp.Problem(spec) as P:
+        good = P.excess_mu(rho)
+        for bad in (-1e-300, np.nan, np.inf):
+            r = rho.copy()
+            r[2, 9, 9, 9] = bad
+            out = np.full_like(r, 7.0)
+            rc = pnp.lib().pnp_excess_mu(P.h, pnp._ptr(r), pnp._ptr(out), -1)
+            assert rc == pnp.ERR_INVALID and (out == 7.0).all()
+            assert P.status() == pnp.OK
+        assert np.array_equal(P.excess_mu(rho), good)
+        zero = np.zeros_like(rho)
+        zero[0, 0, 0, 0] = -0.0
+        assert np.isfinite(P.excess_mu(zero)).all()
+
+
+@pytest.mark.parametrize("species", [1, 3, 5])
+@pytest.mark.parametrize("length", [16, 20, 24, 40, 48, 64, 80, 96])
+def test_wide_z_kernels_match_oracle(pnp, length, species):
+    spec, rho = mu_microbench(shape=(6, 7, length - 4))
+    R, rb = (1.5, 2.0, 3.0, 1.0, 2.5)[:species], (0.004, 0.002, 0.0005, 0.004, 0.001)[:species]
+    spec.R, spec.rho_b, spec.q, spec.depth = R, rb, (1, -1, 0, 1, -1)[:species], (0.0,) * species
+    spec.fft_len = (16, 16, length)
+    rng = np.random.default_rng(length + species)
+    rho = np.stack([r * rng.lognormal(0.0, 0.1, spec.shape) for r in rb])
+    ref, bad = oracle.excess_mu(spec, rho)
+    assert bad == 0
+    with pnp.Problem(spec) as P:
+        for precision in ("fp64", "df64"):
+            mu = P.excess_mu(rho, precision=precision)
+            assert np.abs(mu - ref).max() <= 1e-10 * np.abs(ref).max()
