@@ -83,7 +83,7 @@ void tile_candidates(int G, int axis, std::vector<int> *out) {
     out->assign(1, 0);     // the built-in rule
     if (!G) return;
     if (axis == 0) {
-        for (int thr : {64, 128, 256})
+        for (int thr : {32, 64, 128, 256})
             if (thr / G >= 1) out->push_back(thr / G);
     } else if (axis == 1) {
         for (int tx : {2, 4, 8, 16, 32})

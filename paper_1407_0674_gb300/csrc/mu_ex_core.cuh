@@ -778,10 +778,37 @@ template <auto K> static void ensure_smem() {
 constexpr long kSmemCap = 200 * 1024;
 constexpr int kMaxThreads = 256;
 
-// lines per CTA of the x kernels: the tuned tile if set, else 256 threads;
-// at most 1024 threads, the shared-memory cap and the line pairs there are
-static int x_lines(const Problem *p, int G, long ex_bytes, int npairs) {
-    int P = p->tile[0] > 0 ? p->tile[0] : 256 / G;
+// Threads per CTA of the x and y kernels and columns per CTA of the z kernels,
+// unless tuned.  A line's transform meets at four block barriers, so a CTA
+// should be no larger than its loads need: with 256 threads the FP64 kernels
+// lose 10 to 30 % at the barriers, and double-float at 256 points, which fills
+// its registers, is the one kernel that prefers them.  Measured (us, 256
+// threads -> these): x stages of 70 x 45 x 101 FP64 810 -> 620, of 128^3 -> 256^3
+// FP64 3290 -> 2960 and FP32 411 -> 375; y passes of 128^3 -> 256^3 FP64 5550 ->
+// 4590, of a 96^3 film FP64 742 -> 624.  (Two columns also suit double-float at
+// 256 points, 1200 -> 1125 us, but only while no other call runs: with calls on
+// three streams the step went from 5.47 to 5.61 ms.)
+template <typename T> static int x_threads(int L) {
+    if (std::is_same<T, double>::value) return 64;
+    if (std::is_same<T, float>::value) return L == 256 ? 32 : 64;
+    return L == 256 ? 256 : 128;
+}
+template <typename T> static int y_columns(int L) {
+    if (std::is_same<T, double>::value) return L == 256 ? 2 : (L == 48 ? 8 : 4);
+    if (std::is_same<T, float>::value) return 8;
+    return L == 256 || L == 80 ? 16 : 8;
+}
+// one warp per z CTA at 128 points in FP32 and double-float: a 96^3 film's z MAC
+// and z back take 69 and 86 us for 84 and 113 (FP32), 302 and 291 us for 394 and
+// 386 (double-float)
+template <typename T> static int z_columns(int L, int fits) {
+    return L == 128 && !std::is_same<T, double>::value ? 1 : fits;
+}
+
+// lines per CTA of the x kernels: the tuned tile if set, else x_threads; at most
+// kMaxThreads threads, the shared-memory cap and the line pairs there are
+template <typename T> static int x_lines(const Problem *p, int L, int G, long ex_bytes, int npairs) {
+    int P = p->tile[0] > 0 ? p->tile[0] : std::max(1, x_threads<T>(L) / G);
     P = std::min<long>(P, std::min<long>(kMaxThreads / G, kSmemCap / ex_bytes));
     return std::max(1, std::min(P, npairs));
 }
@@ -913,7 +940,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
     tm.begin(0, st);
     if (!with_shape(d.Lx, [&](auto a, auto b) {
             constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
-            const int P = x_lines(p, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
+            const int P = x_lines<T>(p, d.Lx, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
             ensure_smem<k_xfwd_r<T, N1, N2>>();
             dim3 g((d.npairs + P - 1) / P, d.nz, s);
             k_xfwd_r<T, N1, N2><<<g, P * G, P * Shape<N1, N2>::EX * cs, st>>>(d_rho, N, A, d, twx, P);
@@ -937,7 +964,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
         }
         if (!with_shape(d.Ly, [&](auto a, auto b) {
                 constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
-                int TX = pow2_le(std::min<long>(256 / G, 16));
+                int TX = pow2_le(std::min<long>(256 / G, y_columns<T>(d.Ly)));
                 if (p->tile[1] > 0)
                     TX = std::max(1, std::min<int>(p->tile[1], (int)std::min<long>(kMaxThreads / G,
                                                                                     kSmemCap / (Shape<N1, N2>::EX * (long)cs))));
@@ -979,6 +1006,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
                 // slots (with N1 lanes' worth of them, L = 80 ran 8 warps per SM)
                 const long per_col = ((long)s * N1 * N2 + Shape<N1, N2>::EX) * (long)cs;
                 int TX = pow2_le(std::max<long>(1, std::min<long>(std::min<long>(128 / G, 8), kBudget / (2 * per_col))));
+                TX = z_columns<T>(d.Lz, TX);
                 while (TX > 1 && (long)((d.Wx + TX - 1) / TX) * (d.Ly / 2 + 1) < 2 * 152) TX /= 2;
                 if (p->tile[2] > 0)
                     TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
@@ -1024,7 +1052,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
     if (!with_shape(d.Lx, [&](auto a, auto b) {
             constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
             if (kSplitDerivatives) {
-                const int P = x_lines(p, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
+                const int P = x_lines<T>(p, d.Lx, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
                 const size_t sm = P * Shape<N1, N2>::EX * cs;
                 dim3 g((d.npairs + P - 1) / P, d.nz, kNumWeighted);
                 ensure_smem<k_xinv_raw_r<T, N1, N2, V>>();
@@ -1065,7 +1093,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
     const double *E = p->msa ? p->d_E : nullptr;
     if (!with_shape(d.Lx, [&](auto a, auto b) {
             constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
-            const int P = x_lines(p, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
+            const int P = x_lines<T>(p, d.Lx, G, Shape<N1, N2>::EX * (long)cs, d.npairs);
             ensure_smem<k_xinv_r<T, N1, N2>>();
             dim3 g((d.npairs + P - 1) / P, d.nz, s);
             k_xinv_r<T, N1, N2><<<g, P * G, P * Shape<N1, N2>::EX * cs, st>>>(A, d_mu, N, d, twx, U, sc, P, E);
