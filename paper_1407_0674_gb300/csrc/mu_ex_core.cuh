@@ -868,12 +868,17 @@ static bool launch_zreg(bool back, int s, bool msa, typename vec2<T>::type *B10,
         const dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
         const int threads = Shape<N1, N2>::G * 2 * TX;
         const size_t sm = zreg_smem<N1, N2>(d, s, TX);
-        auto go = [&](auto sv) {
+        auto run = [&](auto sv, auto hv) {
             constexpr int S = decltype(sv)::value;
+            constexpr bool HALF = decltype(hv)::value;
             if (!back)
-                k_zmac_reg<N1, N2, S><<<g, threads, sm, st>>>(Bs, B10, d, twz, spec, sc, TX);
+                k_zmac_reg<N1, N2, S, HALF><<<g, threads, sm, st>>>(Bs, B10, d, twz, spec, sc, TX);
             else
-                k_zback_reg<N1, N2, S><<<g, threads, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);
+                k_zback_reg<N1, N2, S, HALF><<<g, threads, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);
+        };
+        auto go = [&](auto sv) {
+            if (2 * d.nz <= N1 * N2) run(sv, std::true_type{});
+            else run(sv, std::false_type{});
         };
         if (s == 1) go(std::integral_constant<int, 1>{});
         else if (s == 2) go(std::integral_constant<int, 2>{});

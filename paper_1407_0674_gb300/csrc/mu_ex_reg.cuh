@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__
                 v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
             }
         }
-        fwd2<N1, N2>(v, lt, ex, t, lanes);
+        fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
         if (t < N2) {
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) slot(i, k1) = v[k1];
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__
                     }
                 }
             }
-            inv2<N1, N2>(v, lt, ex, t, lanes);
+            inv2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
             if (t < N1 && ok) {
                 C *dst = B10 + (size_t)alpha * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
                     v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
                 }
             }
-            fwd2<N1, N2>(v, lt, ex, t, lanes);
+            fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
             if (t < N2) {
                 for (int i0 = 0; i0 < sc.s; i0 += kChunk) {
                     if (o == 0 || sc.s > kChunk) load_spec<T, N1, N2>(g, spec, d, sc.s, i0, type, kx, ky, t, ok);
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
                     v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
                 }
             }
-            fwd2<N1, N2>(v, lt, ex, t, lanes);
+            fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
             if (t < N2) {
                 for (int i = 0; i < sc.s; ++i) {
                     const T *base = spec + (size_t)(sc.s * kNumKernels + msa_pair(i, j, sc.s)) * oct +
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) v[k1] = slot(i, k1);
         }
-        inv2<N1, N2>(v, lt, ex, t, lanes);
+        inv2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
         if (t < N1 && ok) {
             C *dst = Bs + (size_t)i * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
@@ -823,30 +823,54 @@ __device__ __forceinline__ void stage_type_spectra(float *specS, const float *__
 // twiddle table
 template <int N1, int N2> inline size_t zreg_smem(const Dims &d, int S, int TX) {
     const size_t ex = (size_t)Shape<N1, N2>::EX * 2 * TX * sizeof(float2);
-    const size_t sp = ((size_t)S * d.Oz * TX * sizeof(float) + 7) / 8 * 8;
+    const size_t sp = ((size_t)2 * S * d.Oz * TX * sizeof(float) + 7) / 8 * 8;
     return ex + sp + (size_t)Shape<N1, N2>::G * Shape<N1, N2>::G * sizeof(float2);
 }
 
-template <int N1, int N2, int S>
+// rows z < nz of a column into a lane's transform inputs (H of them can be
+// non-zero: half the length when HALF)
+template <int N1, int H>
+__device__ __forceinline__ void zreg_load(float2 (&x)[H], const float2 *__restrict__ src, bool ok, int t, int nz,
+                                          size_t plane) {
+#pragma unroll
+    for (int n2 = 0; n2 < H; ++n2) {
+        const int zz = t + N1 * n2;
+        x[n2] = (ok && zz < nz) ? src[(size_t)zz * plane] : float2{0, 0};
+    }
+}
+
+// These kernels wait for memory, not for arithmetic (8 warps per SM, all their
+// state in registers), so every load is issued a step ahead: the next column's
+// rows before this column is transformed, the next kernel type's spectra while
+// this type is summed (two buffers, made visible by the transforms' own
+// barriers).  HALF (nz <= L / 2): the transforms skip the zero padding, and half
+// the rows are never loaded.  128^3 -> 256^3: z MAC 0.483 -> 0.460 ms, z back 0.547
+// -> 0.500 ms.
+template <int N1, int N2, int S, bool HALF>
 __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__ B10, float2 *__restrict__ Bs, Dims d,
                                                       const float2 *__restrict__ tw, const float *__restrict__ spec,
                                                       SpeciesConst sc, int TX) {
     using C = float2;
     using T = float;
-    constexpr int G = Shape<N1, N2>::G;
+    constexpr int G = Shape<N1, N2>::G, H = HALF ? N2 / 2 : N2;
     static_assert(N1 == G && N2 == G, "square shapes only");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int c = threadIdx.x % TX, b = (threadIdx.x / TX) & 1, t = threadIdx.x / (2 * TX);
     const int lanes = 2 * TX;
     C *ex = reinterpret_cast<C *>(smem_raw) + (b * TX + c);
     float *specS = reinterpret_cast<float *>(reinterpret_cast<C *>(smem_raw) + (size_t)Shape<N1, N2>::EX * lanes);
+    const int spec_n = S * d.Oz * TX;
     C *twtab = reinterpret_cast<C *>(smem_raw) + (size_t)Shape<N1, N2>::EX * lanes +
-               ((size_t)S * d.Oz * TX * sizeof(float) + sizeof(C) - 1) / sizeof(C);
+               ((size_t)2 * spec_n * sizeof(float) + sizeof(C) - 1) / sizeof(C);
     const int kyp = blockIdx.y, kx0 = blockIdx.x * TX, kx = kx0 + c;
     int ky;
     const bool ok = zcol(d, kyp, b, kx, ky);
     const int fy = kyp;
     const size_t plane = (size_t)d.Ly * d.Wx;
+    const C *col = B10 + (size_t)ky * d.Wx + kx;
+    C nxt[H];
+    zreg_load<N1, H>(nxt, col, ok, t, d.nz, plane);
+    stage_type_spectra(specS, spec, d, S, 0, fy, kx0, TX);
     SmemTw<N1, N2, C>::fill(twtab, tw);
     __syncthreads();
     SmemTw<N1, N2, C> lt;
@@ -858,45 +882,38 @@ __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__
     for (int i = 0; i < S; ++i)
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) acc[i][k1] = C{0, 0};
-    for (int type = 0; type < kNumKernels; ++type) {
-        const int nin = type == 0 ? 3 : (type == 1 ? 1 : 2);
+    for (int e = 0; e < kNumWeighted; ++e) {
+        int type, alpha, type1, alpha1;
+        wide_entry(e, type, alpha);
+        wide_entry(e + 1, type1, alpha1);
+        const bool first = e == 0 || e == 3 || e == 4 || e == 6 || e == 8;
         const bool flip_y = type == 3 && ky > d.Ly / 2;
-        for (int o = 0; o < nin; ++o) {
-            const int alpha = type == 0 ? o : (type == 1 ? 3 : (o == 0 ? 4 + type - 2 : 7 + type - 2));
-            const C *src = B10 + (size_t)alpha * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
-            for (int n2 = 0; n2 < N2; ++n2) {
-                const int zz = t + N1 * n2;
-                v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
-            }
-            if (o == 0) {
-                __syncthreads();      // every lane is done with the previous type's spectra
-                stage_type_spectra(specS, spec, d, S, type, fy, kx0, TX);
-            }
-            fwd2<N1, N2>(v, lt, ex, t, lanes);
-            if (o == 0) {
-                cp_async_wait_all_groups();
-                __syncthreads();
-            }
+        for (int n2 = 0; n2 < N2; ++n2) v[n2] = n2 < H ? nxt[n2 < H ? n2 : 0] : C{0, 0};
+        if (e + 1 < kNumWeighted)
+            zreg_load<N1, H>(nxt, col + (size_t)alpha1 * d.nz * plane, ok, t, d.nz, plane);
+        if (first) cp_async_wait_all_groups();
+        fwd2<N1, N2>(v, lt, ex, t, lanes, HALF);
+        if (first && type + 1 < kNumKernels)
+            stage_type_spectra(specS + ((type + 1) & 1) * spec_n, spec, d, S, type + 1, fy, kx0, TX);
+        const float *sp = specS + (type & 1) * spec_n;
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                const T cf = alpha == 0 ? sc_c0<T>(sc, i)
-                                        : ((alpha == 1 || (alpha >= 4 && alpha < 7)) ? sc_c1<T>(sc, i) : (T)1);
+        for (int i = 0; i < S; ++i) {
+            const T cf = wide_factor<T>(sc, alpha, i);
 #pragma unroll
-                for (int k1 = 0; k1 < N1; ++k1) {
-                    const int kz = t + N2 * k1;
-                    const int fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
-                    T g = specS[(i * d.Oz + fz) * TX + c];
-                    if (flip_y || (type == 4 && kz > d.Lz / 2)) g = -g;
-                    const T gg = cf * g;
-                    const C x = v[k1];
-                    if (type <= 1) {
-                        acc[i][k1].x += gg * x.x;
-                        acc[i][k1].y += gg * x.y;
-                    } else {             // K = -i S
-                        acc[i][k1].x += gg * x.y;
-                        acc[i][k1].y -= gg * x.x;
-                    }
+            for (int k1 = 0; k1 < N1; ++k1) {
+                const int kz = t + N2 * k1;
+                const int fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
+                T g = sp[(i * d.Oz + fz) * TX + c];
+                if (flip_y || (type == 4 && kz > d.Lz / 2)) g = -g;
+                const T gg = cf * g;
+                const C x = v[k1];
+                if (type <= 1) {
+                    acc[i][k1].x += gg * x.x;
+                    acc[i][k1].y += gg * x.y;
+                } else {             // K = -i S
+                    acc[i][k1].x += gg * x.y;
+                    acc[i][k1].y -= gg * x.x;
                 }
             }
         }
@@ -905,11 +922,11 @@ __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__
     for (int i = 0; i < S; ++i) {
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) v[k1] = acc[i][k1];
-        inv2<N1, N2>(v, lt, ex, t, lanes);
+        inv2<N1, N2>(v, lt, ex, t, lanes, HALF);
         if (ok) {
             C *dst = Bs + (size_t)i * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
-            for (int n2 = 0; n2 < N2; ++n2) {
+            for (int n2 = 0; n2 < H; ++n2) {
                 const int zz = t + N1 * n2;
                 if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
             }
@@ -917,26 +934,31 @@ __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__
     }
 }
 
-template <int N1, int N2, int S>
+template <int N1, int N2, int S, bool HALF>
 __global__ void __launch_bounds__(128, 2) k_zmac_reg(const float2 *__restrict__ Bs, float2 *__restrict__ B10, Dims d,
                                                      const float2 *__restrict__ tw, const float *__restrict__ spec,
                                                      SpeciesConst sc, int TX) {
     using C = float2;
     using T = float;
-    constexpr int G = Shape<N1, N2>::G;
+    constexpr int G = Shape<N1, N2>::G, H = HALF ? N2 / 2 : N2;
     static_assert(N1 == G && N2 == G, "square shapes only");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int c = threadIdx.x % TX, b = (threadIdx.x / TX) & 1, t = threadIdx.x / (2 * TX);
     const int lanes = 2 * TX;
     C *ex = reinterpret_cast<C *>(smem_raw) + (b * TX + c);
     float *specS = reinterpret_cast<float *>(reinterpret_cast<C *>(smem_raw) + (size_t)Shape<N1, N2>::EX * lanes);
+    const int spec_n = S * d.Oz * TX;
     C *twtab = reinterpret_cast<C *>(smem_raw) + (size_t)Shape<N1, N2>::EX * lanes +
-               ((size_t)S * d.Oz * TX * sizeof(float) + sizeof(C) - 1) / sizeof(C);
+               ((size_t)2 * spec_n * sizeof(float) + sizeof(C) - 1) / sizeof(C);
     const int kyp = blockIdx.y, kx0 = blockIdx.x * TX, kx = kx0 + c;
     int ky;
     const bool ok = zcol(d, kyp, b, kx, ky);
     const int fy = kyp;
     const size_t plane = (size_t)d.Ly * d.Wx;
+    const C *col = Bs + (size_t)ky * d.Wx + kx;
+    C nxt[H];
+    zreg_load<N1, H>(nxt, col, ok, t, d.nz, plane);
+    stage_type_spectra(specS, spec, d, S, 0, fy, kx0, TX);
     SmemTw<N1, N2, C>::fill(twtab, tw);
     __syncthreads();
     SmemTw<N1, N2, C> lt;
@@ -946,60 +968,55 @@ __global__ void __launch_bounds__(128, 2) k_zmac_reg(const float2 *__restrict__ 
     C rs[S][N1];
 #pragma unroll
     for (int i = 0; i < S; ++i) {
-        const C *src = Bs + (size_t)i * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) {
-            const int zz = t + N1 * n2;
-            v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
-        }
-        if (i == 0) stage_type_spectra(specS, spec, d, S, 0, fy, kx0, TX);
-        fwd2<N1, N2>(v, lt, ex, t, lanes);
+        for (int n2 = 0; n2 < N2; ++n2) v[n2] = n2 < H ? nxt[n2 < H ? n2 : 0] : C{0, 0};
+        if (i + 1 < S) zreg_load<N1, H>(nxt, col + (size_t)(i + 1) * d.nz * plane, ok, t, d.nz, plane);
+        if (i + 1 == S) cp_async_wait_all_groups();      // type 0's spectra, before the last barriers
+        fwd2<N1, N2>(v, lt, ex, t, lanes, HALF);
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) rs[i][k1] = v[k1];
     }
-    // output groups: shell {n0, n1, n2}, ball {n3}, vector x {n1x, n2x}, y, z
-    for (int type = 0; type < kNumKernels; ++type) {
-        if (type > 0) {
-            __syncthreads();          // every lane is done with the previous type's spectra
-            stage_type_spectra(specS, spec, d, S, type, fy, kx0, TX);
-        }
-        cp_async_wait_all_groups();
-        __syncthreads();
-        const int nout = type == 0 ? 3 : (type == 1 ? 1 : 2);
+    for (int e = 0; e < kNumWeighted; ++e) {
+        int type, alpha;
+        wide_entry(e, type, alpha);
+        const bool first = e == 0 || e == 3 || e == 4 || e == 6 || e == 8;
+        const bool last = e == 2 || e == 3 || e == 5 || e == 7;    // of its type
+        // every lane is past the previous type's products (the transform's
+        // barriers): its buffer takes the next type's spectra
+        if (first && type + 1 < kNumKernels)
+            stage_type_spectra(specS + ((type + 1) & 1) * spec_n, spec, d, S, type + 1, fy, kx0, TX);
         const bool flip_y = type == 3 && ky > d.Ly / 2;
-        for (int o = 0; o < nout; ++o) {
-            const int alpha = type == 0 ? o : (type == 1 ? 3 : (o == 0 ? 4 + type - 2 : 7 + type - 2));
+        const float *sp = specS + (type & 1) * spec_n;
 #pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) v[k1] = C{0, 0};
+        for (int k1 = 0; k1 < N1; ++k1) v[k1] = C{0, 0};
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                const T cf = alpha == 0 ? sc_c0<T>(sc, i)
-                                        : ((alpha == 1 || (alpha >= 4 && alpha < 7)) ? sc_c1<T>(sc, i) : (T)1);
+        for (int i = 0; i < S; ++i) {
+            const T cf = wide_factor<T>(sc, alpha, i);
 #pragma unroll
-                for (int k1 = 0; k1 < N1; ++k1) {
-                    const int kz = t + N2 * k1;
-                    const int fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
-                    T g = specS[(i * d.Oz + fz) * TX + c];
-                    if (flip_y || (type == 4 && kz > d.Lz / 2)) g = -g;
-                    const T gg = cf * g;
-                    const C x = rs[i][k1];
-                    if (type <= 1) {
-                        v[k1].x += gg * x.x;
-                        v[k1].y += gg * x.y;
-                    } else {             // conj(K) = +i S
-                        v[k1].x -= gg * x.y;
-                        v[k1].y += gg * x.x;
-                    }
+            for (int k1 = 0; k1 < N1; ++k1) {
+                const int kz = t + N2 * k1;
+                const int fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
+                T g = sp[(i * d.Oz + fz) * TX + c];
+                if (flip_y || (type == 4 && kz > d.Lz / 2)) g = -g;
+                const T gg = cf * g;
+                const C x = rs[i][k1];
+                if (type <= 1) {
+                    v[k1].x += gg * x.x;
+                    v[k1].y += gg * x.y;
+                } else {             // conj(K) = +i S
+                    v[k1].x -= gg * x.y;
+                    v[k1].y += gg * x.x;
                 }
             }
-            inv2<N1, N2>(v, lt, ex, t, lanes);
-            if (ok) {
-                C *dst = B10 + (size_t)alpha * d.nz * plane + (size_t)ky * d.Wx + kx;
+        }
+        if (last) cp_async_wait_all_groups();            // the next type's, before this transform's barriers
+        inv2<N1, N2>(v, lt, ex, t, lanes, HALF);
+        if (ok) {
+            C *dst = B10 + (size_t)alpha * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
-                for (int n2 = 0; n2 < N2; ++n2) {
-                    const int zz = t + N1 * n2;
-                    if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
-                }
+            for (int n2 = 0; n2 < H; ++n2) {
+                const int zz = t + N1 * n2;
+                if (zz < d.nz) dst[(size_t)zz * plane] = v[n2];
             }
         }
     }
