@@ -821,6 +821,16 @@ static void op_setup(Lane *g, bool faces, cudaStream_t st) {
         k_tail_setup<<<1, kTailThreads, 0, st>>>(tail_args(g, shift, nullptr, nullptr), faces ? 1 : 0);
 }
 
+// one colour sweep (see k_sweep); res: also the swept points' residuals
+static void sweep(cudaStream_t st, const Op &A, const double *xo, const double *xs, double *xw, const double *b, int c,
+                  double *res) {
+    const int G = blocks_for(A.nt, kSweepThreads);
+    if (A.unit && res) k_sweep<true, true><<<G, kSweepThreads, 0, st>>>(A, xo, xs, xw, b, c, res);
+    else if (A.unit) k_sweep<true, false><<<G, kSweepThreads, 0, st>>>(A, xo, xs, xw, b, c, res);
+    else if (res) k_sweep<false, true><<<G, kSweepThreads, 0, st>>>(A, xo, xs, xw, b, c, res);
+    else k_sweep<false, false><<<G, kSweepThreads, 0, st>>>(A, xo, xs, xw, b, c, res);
+}
+
 // x = M b, one V(2,2) cycle on the current operator, from the start values
 // that the kernel producing b left in x (red: b / diag, black: 0).  On level 0
 // x = z, b = r, and the block sums of b . x go to `part`; returns their number.
@@ -834,17 +844,24 @@ static int vcycle(Lane *g, cudaStream_t st, double *part) {
     for (int l = 0; l < g->lt; ++l) {
         Level &L = g->lv[l], &C = g->lv[l + 1];
         const Op A = op_of(L, g->shift);
-        const int G = blocks_for(A.nt, kSweepThreads);
         double *x = xof(l), *y = x2of(l);
         const double *b = bof(l);
         // odd levels: red starts in y, black in x; every sweep writes the
         // buffer its colour is not in, and all end in x
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, x, y, b, 1);
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, y, x, b, 0);
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, y, x, b, 1);
+        sweep(st, A, y, x, y, b, 1, nullptr);
+        sweep(st, A, y, y, x, b, 0, nullptr);
+        // level 0 keeps the black residuals in Ap, idle during the cycle
+        double *known = l == 0 && !L.odd && L.fx == 2 ? g->Ap : nullptr;
+        sweep(st, A, x, y, x, b, 1, known);
         const size_t sm = sizeof(double) * kRestrictCells * L.fx * L.fy * L.fz;
-        k_residual_restrict<<<blocks_for(C.n, kRestrictCells), 256, sm, st>>>(
-            A, x, b, L.fx, L.fy, L.fz, op_of(C, g->shift), C.b, C.x2, C.x);
+        const int R = blocks_for(C.n, kRestrictCells);
+        const Op c = op_of(C, g->shift);
+        if (known && A.unit)
+            k_residual_restrict_red<true><<<R, 128, sm, st>>>(A, x, b, known, L.fy, L.fz, c, C.b, C.x2, C.x);
+        else if (known)
+            k_residual_restrict_red<false><<<R, 128, sm, st>>>(A, x, b, known, L.fy, L.fz, c, C.b, C.x2, C.x);
+        else
+            k_residual_restrict<<<R, 256, sm, st>>>(A, x, b, L.fx, L.fy, L.fz, c, C.b, C.x2, C.x);
     }
     if (g->tail) {
         k_tail<<<1, kTailThreads, g->tail_smem, st>>>(tail_args(g, g->shift, bof(g->lt), xof(g->lt)));
@@ -868,13 +885,15 @@ static int vcycle(Lane *g, cudaStream_t st, double *part) {
         const double *b = bof(l);
         k_prolong_add<<<G, kSweepThreads, 0, st>>>(A, x, FastDiv(L.fx), FastDiv(L.fy), FastDiv(L.fz), C.nx, C.ny, C.x,
                                                    kCoarseScale);
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, x, y, b, 1);
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, x, y, b, 0);
-        k_sweep<<<G, kSweepThreads, 0, st>>>(A, y, y, x, b, 1);
+        sweep(st, A, x, x, y, b, 1, nullptr);
+        sweep(st, A, y, x, y, b, 0, nullptr);
+        sweep(st, A, y, y, x, b, 1, nullptr);
         if (l > 0 || !fuse_dot) {
-            k_sweep<<<G, kSweepThreads, 0, st>>>(A, x, y, x, b, 0);
+            sweep(st, A, x, y, x, b, 0, nullptr);
+        } else if (A.unit) {
+            k_sweep_dot<true><<<nb, 128, 0, st>>>(A, x, y, x, b, part);
         } else {
-            k_sweep_dot<<<nb, 128, 0, st>>>(A, x, y, x, b, part);
+            k_sweep_dot<false><<<nb, 128, 0, st>>>(A, x, y, x, b, part);
         }
     }
     if (!fuse_dot) k_dot<<<nb, 256, 0, st>>>(g->r, g->z, (unsigned)n0, part);
@@ -919,7 +938,8 @@ static cudaError_t pcg_capture(Lane *g, double *x, const double *b, double tol, 
     double *r = g->r, *z = g->z, *z2 = g->z2, *p = g->pv, *Ap = g->Ap;
     double *part_bb = g->partial, *part_rr = part_bb + kDotBlocks, *part_rz = part_rr + kDotBlocks,
            *part_pap = part_rz + kDotBlocks;
-    k_pcg_start<<<NB, 256, 0, st>>>(A, x, b, r, z2, z, part_bb, part_rr);
+    if (A.unit) k_pcg_start<true><<<NB, 256, 0, st>>>(A, x, b, r, z2, z, part_bb, part_rr);
+    else k_pcg_start<false><<<NB, 256, 0, st>>>(A, x, b, r, z2, z, part_bb, part_rr);
     cudaStreamCaptureStatus cs;
     cudaGraph_t cg = nullptr;
     cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &cg, nullptr, nullptr, nullptr);
@@ -935,7 +955,8 @@ static cudaError_t pcg_capture(Lane *g, double *x, const double *b, double tol, 
     if (e != cudaSuccess) return e;
     const int nrz = vcycle(g, sb, part_rz);
     k_pcg_direction<<<NB, 256, 0, sb>>>(p, z, g->ctl, part_rz, nrz, A.n);
-    k_pcg_apply<<<NB, 256, 0, sb>>>(A, p, Ap, part_pap);
+    if (A.unit) k_pcg_apply<true><<<NB, 256, 0, sb>>>(A, p, Ap, part_pap);
+    else k_pcg_apply<false><<<NB, 256, 0, sb>>>(A, p, Ap, part_pap);
     k_pcg_update<<<NB, 256, 0, sb>>>(A, x, r, p, Ap, z2, z, g->ctl, part_pap, NB, part_rr);
     k_pcg_check<<<1, 128, 0, sb>>>(g->ctl, part_rr, NB, maxit, stats, flag, h);
     return cudaStreamEndCapture(sb, &body);
@@ -948,6 +969,7 @@ static void set_operator(Lane *g, bool poisson) {
             std::swap(L.cy, L.pcy);
             std::swap(L.cz, L.pcz);
             std::swap(L.czlo, L.pczlo);
+            std::swap(L.unit, L.punit);
         }
     }
 }
@@ -977,6 +999,8 @@ int gummel_setup(Problem *p) {
         bool last = L.n <= 8 || (L.fx == 1 && L.fy == 1 && L.fz == 1) || first.lv.size() >= 16;
         if (last) L.fx = L.fy = L.fz = 1;
         L.odd = (p->bc[0] == PNP_BC_PERIODIC && nx % 2) || (p->bc[1] == PNP_BC_PERIODIC && ny % 2);
+        // the finest Poisson faces are 1 but for no-flux walls
+        L.punit = first.lv.empty() && p->bc[0] == PNP_BC_PERIODIC && p->bc[1] == PNP_BC_PERIODIC;
         first.lv.push_back(L);
         if (last) break;
         nx /= L.fx; ny /= L.fy; nz /= L.fz;

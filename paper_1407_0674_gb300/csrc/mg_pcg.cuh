@@ -58,6 +58,8 @@ struct Level {
     double *dgn, *idg;             // assembled diagonal and reciprocal of the current operator
     double *x, *b;
     double *x2;                    // second iterate buffer of odd levels (x otherwise)
+    bool punit;                    // every face of the Poisson operator is 1 (level 0, x and y periodic)
+    bool unit;                     // and of the current operator
 };
 
 // what the level kernels read, by value
@@ -69,6 +71,7 @@ struct Op {
     const double *dg;              // optional extra diagonal (Poisson-Boltzmann screening)
     const double *dgn, *idg;
     int odd;
+    int unit;                      // every face is 1: kernels compiled for it do not read them
 };
 
 constexpr int kCoarseSweeps = 40;
@@ -98,6 +101,7 @@ static Op op_of(const Level &L, bool shift = false) {
     A.dg = shift ? L.dg : nullptr;
     A.dgn = L.dgn; A.idg = L.idg;
     A.odd = L.odd ? 1 : 0;
+    A.unit = L.unit ? 1 : 0;
     return A;
 }
 
@@ -138,13 +142,22 @@ __device__ __forceinline__ double op_diag(const Op &A, const Pt &q) {
     return d;
 }
 
-// sum_faces c u_nbr.  `wrap` serves the neighbours across an x or y wrap of
+// sum_faces c u_nbr; UNIT: every c is 1, where the same sums are plain additions
+// (fma(1, a, 1 b) = a + b): six operations instead of eight and no faces to read.
+// `wrap` serves the neighbours across an x or y wrap of
 // odd extent (they have the point's own colour), u all others.
+template <bool UNIT = false>
 __device__ __forceinline__ double op_nbr(const Op &A, const double *u, const double *wrap, const Pt &q) {
     const unsigned xp = nbr_xp(A, q), xm = nbr_xm(A, q), yp = nbr_yp(A, q), ym = nbr_ym(A, q);
     const bool ox = A.odd && (A.nx & 1), oy = A.odd && (A.ny & 1);
     const double *uxp = ox && q.i + 1 == A.nx ? wrap : u, *uxm = ox && q.i == 0 ? wrap : u;
     const double *uyp = oy && q.j + 1 == A.ny ? wrap : u, *uym = oy && q.j == 0 ? wrap : u;
+    if constexpr (UNIT) {
+        double s = (uxp[xp] + uxm[xm]) + (uyp[yp] + uym[ym]);
+        if (q.k + 1 < A.nz) s += u[q.p + A.plane];
+        if (q.k > 0) s += u[q.p - A.plane];
+        return s;
+    }
     const double sx = fma(A.cx[q.p], uxp[xp], A.cx[xm] * uxm[xm]);
     const double sy = fma(A.cy[q.p], uyp[yp], A.cy[ym] * uym[ym]);
     double s = sx + sy;
@@ -163,8 +176,9 @@ __device__ __forceinline__ double quotient(double v, double d, double y) {
 }
 
 // b - (A u)_p
+template <bool UNIT = false>
 __device__ __forceinline__ double op_residual(const Op &A, const double *u, const Pt &q, double b) {
-    return b - (__dmul_rn(A.dgn[q.p], u[q.p]) - op_nbr(A, u, u, q));
+    return b - (__dmul_rn(A.dgn[q.p], u[q.p]) - op_nbr<UNIT>(A, u, u, q));
 }
 
 // ---------------------------------------------------------------------------
@@ -303,18 +317,28 @@ __global__ void k_diag(Op A, double *__restrict__ dgn, double *__restrict__ idg)
 // FP64-bound, and 128-thread CTAs put the 512 warps of a 32^3 colour on 128 SMs,
 // one warp on each quarter of an SM.  With the rest of this file a CG iteration
 // went from 343 to 103 us at 32^3 and from 700 to 290 us at 96^3.
+//
+// RES: the residual of the swept points is written too.  Their neighbours do not
+// change before the restriction, so the sum just formed serves it: three more
+// operations here against ten there.
+template <bool UNIT, bool RES>
 __global__ void __launch_bounds__(kSweepThreads) k_sweep(Op A, const double *xo, const double *xs, double *xw,
-                                                         const double *__restrict__ b, int c) {
+                                                         const double *__restrict__ b, int c,
+                                                         double *__restrict__ res) {
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= A.nt) return;
     const Pt q = pt_colour(A, t, c);
     if (q.i >= A.nx) return;
-    xw[q.p] = quotient(b[q.p] + op_nbr(A, xo, xs, q), A.dgn[q.p], A.idg[q.p]);
+    const double s = op_nbr<UNIT>(A, xo, xs, q), bp = b[q.p], d = A.dgn[q.p];
+    const double v = quotient(bp + s, d, A.idg[q.p]);
+    xw[q.p] = v;
+    if (RES) res[q.p] = bp - (__dmul_rn(d, v) - s);
 }
 
 // the last red sweep of the cycle on level 0 with the block sums of b . x, for
 // even nx and at most 512 x 256 points: thread m owns the pair of slots
 // (2m, 2m + 1), one red point and one black
+template <bool UNIT>
 __global__ void __launch_bounds__(128) k_sweep_dot(Op A, const double *xo, const double *xs, double *xw,
                                                    const double *__restrict__ b, double *__restrict__ part) {
     __shared__ double sh[256];
@@ -326,7 +350,7 @@ __global__ void __launch_bounds__(128) k_sweep_dot(Op A, const double *xo, const
         q.i += up;
         q.p += up;
         const double br = b[q.p];
-        const double v = quotient(br + op_nbr(A, xo, xs, q), A.dgn[q.p], A.idg[q.p]);
+        const double v = quotient(br + op_nbr<UNIT>(A, xo, xs, q), A.dgn[q.p], A.idg[q.p]);
         const double dr = br * v;
         const unsigned pb = p0 + 1 - up;
         const double db = b[pb] * xo[pb];
@@ -366,6 +390,38 @@ __global__ void __launch_bounds__(256) k_residual_restrict(Op F, const double *_
     if (threadIdx.x >= kRestrictCells || q >= C.n) return;
     double s = res[threadIdx.x];
     for (int k = 1; k < nch; ++k) s += res[k * kRestrictCells + threadIdx.x];
+    const Pt Q = pt_flat(C, q);
+    bc[q] = s;
+    if ((Q.i + Q.j + Q.k) & 1) xblack[q] = 0.0;
+    else xred[q] = quotient(s, C.dgn[q], C.idg[q]);
+}
+
+// The same on an even level with fx = 2 whose black residuals k_sweep left in
+// `known`: of each pair of children along x the red one is computed, on full
+// warps, and the black one read.
+template <bool UNIT>
+__global__ void __launch_bounds__(128) k_residual_restrict_red(Op F, const double *__restrict__ x,
+                                                               const double *__restrict__ b,
+                                                               const double *__restrict__ known, int fy, int fz, Op C,
+                                                               double *__restrict__ bc, double *__restrict__ xred,
+                                                               double *__restrict__ xblack) {
+    extern __shared__ double res[];                   // [child][cell], child = 2 (c fy + b) + a
+    const int rows = fy * fz;
+    for (int e = threadIdx.x; e < rows * kRestrictCells; e += blockDim.x) {
+        const int row = e / kRestrictCells, cell = e % kRestrictCells;
+        const unsigned q = blockIdx.x * kRestrictCells + cell;
+        if (q >= C.n) continue;
+        const Pt Q = pt_flat(C, q);
+        const int j = Q.j * fy + row % fy, k = Q.k * fz + row / fy, a = (j + k) & 1;
+        Pt f{2 * Q.i + a, j, k, ((unsigned)k * F.ny + j) * F.nx + 2 * Q.i + a};
+        res[(2 * row + a) * kRestrictCells + cell] = op_residual<UNIT>(F, x, f, b[f.p]);
+        res[(2 * row + 1 - a) * kRestrictCells + cell] = known[f.p + 1 - 2 * a];
+    }
+    __syncthreads();
+    const unsigned q = blockIdx.x * kRestrictCells + threadIdx.x;
+    if (threadIdx.x >= kRestrictCells || q >= C.n) return;
+    double s = res[threadIdx.x];
+    for (int k = 1; k < 2 * rows; ++k) s += res[k * kRestrictCells + threadIdx.x];
     const Pt Q = pt_flat(C, q);
     bc[q] = s;
     if ((Q.i + Q.j + Q.k) & 1) xblack[q] = 0.0;
@@ -455,6 +511,7 @@ __global__ void __launch_bounds__(256) k_dot(const double *__restrict__ a, const
 // start values, and the loop decision.
 
 // r = b - A x, the cycle's start values, and the partials of b . b and r . r
+template <bool UNIT>
 __global__ void __launch_bounds__(256) k_pcg_start(Op A, const double *__restrict__ x, const double *__restrict__ b,
                                                    double *__restrict__ r, double *__restrict__ zred,
                                                    double *__restrict__ zblack, double *__restrict__ part_bb,
@@ -463,7 +520,7 @@ __global__ void __launch_bounds__(256) k_pcg_start(Op A, const double *__restric
     for (unsigned p = blockIdx.x * 256 + threadIdx.x; p < A.n; p += gridDim.x * 256) {
         const Pt q = pt_flat(A, p);
         const double bp = b[p];
-        const double v = op_residual(A, x, q, bp);
+        const double v = op_residual<UNIT>(A, x, q, bp);
         r[p] = v;
         if ((q.i + q.j + q.k) & 1) zblack[p] = 0.0;
         else zred[p] = quotient(v, A.dgn[p], A.idg[p]);
@@ -492,12 +549,13 @@ __global__ void __launch_bounds__(256) k_pcg_direction(double *__restrict__ p, c
 }
 
 // Ap = A p and the partials of p . Ap
+template <bool UNIT>
 __global__ void __launch_bounds__(256) k_pcg_apply(Op A, const double *__restrict__ p, double *__restrict__ Ap,
                                                    double *__restrict__ part) {
     double acc = 0.0;
     for (unsigned k = blockIdx.x * 256 + threadIdx.x; k < A.n; k += gridDim.x * 256) {
         const double u = p[k];
-        const double v = fma(A.dgn[k], u, -op_nbr(A, p, p, pt_flat(A, k)));
+        const double v = fma(A.dgn[k], u, -op_nbr<UNIT>(A, p, p, pt_flat(A, k)));
         Ap[k] = v;
         acc = fma(u, v, acc);
     }
