@@ -314,7 +314,7 @@ __global__ void k_xfwd(const double *__restrict__ in, size_t in_fstride, typenam
     const int pair0 = blockIdx.x * P;
     const double *src = in + f * in_fstride + (size_t)z * d.ny * d.nx;
     for (int idx = threadIdx.x; idx < P * d.Lx; idx += blockDim.x) {
-        const int p = idx / d.Lx, x = idx % d.Lx;
+        const int p = fdiv(idx, ax.mgL), x = idx - p * d.Lx;
         const int y0 = 2 * (pair0 + p);
         T re = 0, im = 0;
         if (x < d.nx && y0 < d.ny) {
@@ -327,7 +327,7 @@ __global__ void k_xfwd(const double *__restrict__ in, size_t in_fstride, typenam
     C *r = fft_lines<false>(a, b, P, ax, tw);
     C *dst = A + ((size_t)f * d.nz + z) * d.ny * d.Wx;
     for (int idx = threadIdx.x; idx < P * d.Wx; idx += blockDim.x) {
-        const int p = idx / d.Wx, k = idx % d.Wx;
+        const int p = fdiv(idx, ax.mgW), k = idx - p * d.Wx;
         const int y0 = 2 * (pair0 + p);
         if (y0 >= d.ny) continue;
         C zk = r[k * P + p];
@@ -352,10 +352,10 @@ __global__ void k_ypass(const typename vec2<T>::type *__restrict__ in, typename 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + (size_t)TX * d.Ly;
-    const int z = blockIdx.y, f = blockIdx.z, kx0 = blockIdx.x * TX;
+    const int z = blockIdx.y, f = blockIdx.z, kx0 = blockIdx.x * TX, sh = 31 - __clz(TX);
     const C *src = in + ((size_t)f * d.nz + z) * rows_in * d.Wx;
     for (int idx = threadIdx.x; idx < TX * d.Ly; idx += blockDim.x) {
-        const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+        const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
         C v = C{0, 0};
         if (j < n_in && kx < d.Wx) v = src[(size_t)j * d.Wx + kx];
         a[j * TX + c] = v;
@@ -364,7 +364,7 @@ __global__ void k_ypass(const typename vec2<T>::type *__restrict__ in, typename 
     C *r = fft_lines<INV>(a, b, TX, ax, tw);
     C *dst = out + ((size_t)f * d.nz + z) * rows_out * d.Wx;
     for (int idx = threadIdx.x; idx < TX * n_out; idx += blockDim.x) {
-        const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+        const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
         if (kx < d.Wx) dst[(size_t)j * d.Wx + kx] = r[j * TX + c];
     }
 }
@@ -383,12 +383,12 @@ __global__ void k_zmac(const typename vec2<T>::type *__restrict__ Bs, typename v
     C *rho = reinterpret_cast<C *>(smem_raw);   // s columns
     C *work = rho + (size_t)sc.s * col;
     C *scr = work + col;
-    const int ky = blockIdx.y, kx0 = blockIdx.x * TX;
+    const int ky = blockIdx.y, kx0 = blockIdx.x * TX, sh = 31 - __clz(TX);   // TX: a power of two
     for (int i = 0; i < sc.s; ++i) {
         const C *src = Bs + (size_t)i * d.nz * d.Ly * d.Wx + (size_t)ky * d.Wx;
         C *dst = rho + (size_t)i * col;
         for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-            const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             C v = C{0, 0};
             if (j < d.nz && kx < d.Wx) v = src[(size_t)j * d.Ly * d.Wx + kx];
             dst[idx] = v;
@@ -398,7 +398,7 @@ __global__ void k_zmac(const typename vec2<T>::type *__restrict__ Bs, typename v
     }
     for (int alpha = 0; alpha < kNumWeighted; ++alpha) {
         for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-            const int kz = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int kz = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             C acc = C{0, 0};
             if (kx < d.Wx) {
                 for (int i = 0; i < sc.s; ++i) {
@@ -425,7 +425,7 @@ __global__ void k_zmac(const typename vec2<T>::type *__restrict__ Bs, typename v
         C *r = fft_lines<true>(work, scr, TX, ax, tw);
         C *dst = B10 + (size_t)alpha * d.nz * d.Ly * d.Wx + (size_t)ky * d.Wx;
         for (int idx = threadIdx.x; idx < TX * d.nz; idx += blockDim.x) {
-            const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             if (kx < d.Wx) dst[(size_t)j * d.Ly * d.Wx + kx] = r[idx];
         }
         __syncthreads();
@@ -451,7 +451,7 @@ __global__ void k_xfused(typename vec2<T>::type *__restrict__ A, Dims d, FftAxis
         C *buf = fld + (size_t)alpha * line;
         const C *src = base + alpha * fstride;
         for (int idx = threadIdx.x; idx < line; idx += blockDim.x) {
-            const int p = idx / d.Lx, k = idx % d.Lx;
+            const int p = fdiv(idx, ax.mgL), k = idx - p * d.Lx;
             const int y0 = 2 * (pair0 + p);
             C Z = C{0, 0};
             if (y0 < d.ny) {
@@ -470,7 +470,7 @@ __global__ void k_xfused(typename vec2<T>::type *__restrict__ A, Dims d, FftAxis
     // pointwise derivatives; line y0 in .x, line y0+1 in .y
     int bad = 0;
     for (int idx = threadIdx.x; idx < line; idx += blockDim.x) {
-        const int p = idx / d.Lx, x = idx % d.Lx;
+        const int p = fdiv(idx, ax.mgL), x = idx - p * d.Lx;
         const int y0 = 2 * (pair0 + p);
         for (int h = 0; h < 2; ++h) {
             const int y = y0 + h;
@@ -498,7 +498,7 @@ __global__ void k_xfused(typename vec2<T>::type *__restrict__ A, Dims d, FftAxis
         C *r = fft_lines<false>(buf, scr, P, ax, tw);
         C *dst = base + alpha * fstride;
         for (int idx = threadIdx.x; idx < P * d.Wx; idx += blockDim.x) {
-            const int p = idx / d.Wx, k = idx % d.Wx;
+            const int p = fdiv(idx, ax.mgW), k = idx - p * d.Wx;
             const int y0 = 2 * (pair0 + p);
             if (y0 >= d.ny) continue;
             C zk = r[k * P + p];
@@ -525,12 +525,12 @@ __global__ void k_zback(const typename vec2<T>::type *__restrict__ B10, typename
     C *acc = reinterpret_cast<C *>(smem_raw);   // s accumulators
     C *work = acc + (size_t)sc.s * col;
     C *scr = work + col;
-    const int ky = blockIdx.y, kx0 = blockIdx.x * TX;
+    const int ky = blockIdx.y, kx0 = blockIdx.x * TX, sh = 31 - __clz(TX);   // TX: a power of two
     for (int idx = threadIdx.x; idx < sc.s * col; idx += blockDim.x) acc[idx] = C{0, 0};
     for (int alpha = 0; alpha < kNumWeighted; ++alpha) {
         const C *src = B10 + (size_t)alpha * d.nz * d.Ly * d.Wx + (size_t)ky * d.Wx;
         for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-            const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             C v = C{0, 0};
             if (j < d.nz && kx < d.Wx) v = src[(size_t)j * d.Ly * d.Wx + kx];
             work[idx] = v;
@@ -538,7 +538,7 @@ __global__ void k_zback(const typename vec2<T>::type *__restrict__ B10, typename
         __syncthreads();
         C *r = fft_lines<false>(work, scr, TX, ax, tw);
         for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-            const int kz = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int kz = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             if (kx >= d.Wx) continue;
             const C v = r[idx];
             for (int i = 0; i < sc.s; ++i) {
@@ -569,7 +569,7 @@ __global__ void k_zback(const typename vec2<T>::type *__restrict__ B10, typename
         for (int j = 0; j < sc.s; ++j) {
             const C *src = Bs + (size_t)j * d.nz * d.Ly * d.Wx + (size_t)ky * d.Wx;
             for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-                const int z = idx / TX, c = idx % TX, kx = kx0 + c;
+                const int z = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
                 C v = C{0, 0};
                 if (z < d.nz && kx < d.Wx) v = src[(size_t)z * d.Ly * d.Wx + kx];
                 work[idx] = v;
@@ -577,7 +577,7 @@ __global__ void k_zback(const typename vec2<T>::type *__restrict__ B10, typename
             __syncthreads();
             C *r = fft_lines<false>(work, scr, TX, ax, tw);
             for (int idx = threadIdx.x; idx < col; idx += blockDim.x) {
-                const int kz = idx / TX, c = idx % TX, kx = kx0 + c;
+                const int kz = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
                 if (kx >= d.Wx) continue;
                 const int fz = kz <= d.Lz / 2 ? kz : d.Lz - kz;
                 const C v = r[idx];
@@ -596,7 +596,7 @@ __global__ void k_zback(const typename vec2<T>::type *__restrict__ B10, typename
         C *r = fft_lines<true>(acc + (size_t)i * col, work, TX, ax, tw);
         C *dst = Bs + (size_t)i * d.nz * d.Ly * d.Wx + (size_t)ky * d.Wx;
         for (int idx = threadIdx.x; idx < TX * d.nz; idx += blockDim.x) {
-            const int j = idx / TX, c = idx % TX, kx = kx0 + c;
+            const int j = idx >> sh, c = idx & (TX - 1), kx = kx0 + c;
             if (kx < d.Wx) dst[(size_t)j * d.Ly * d.Wx + kx] = r[idx];
         }
         __syncthreads();
@@ -617,7 +617,7 @@ __global__ void k_xinv(const typename vec2<T>::type *__restrict__ A, double *__r
     const int z = blockIdx.y, f = blockIdx.z, pair0 = blockIdx.x * P;
     const C *src = A + ((size_t)f * d.nz + z) * d.ny * d.Wx;
     for (int idx = threadIdx.x; idx < P * d.Lx; idx += blockDim.x) {
-        const int p = idx / d.Lx, k = idx % d.Lx;
+        const int p = fdiv(idx, ax.mgL), k = idx - p * d.Lx;
         const int y0 = 2 * (pair0 + p);
         C Z = C{0, 0};
         if (y0 < d.ny) {

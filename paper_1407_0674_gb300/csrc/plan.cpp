@@ -40,6 +40,13 @@ FftAxis make_axis(int L) {
     for (int p : {2, 3, 5})
         while (m % p == 0) { a.radix[k++] = p; m /= p; }
     a.nst = k;
+    auto magic = [](unsigned n) { return n > 1 ? (unsigned)(((1ull << 32) + n - 1) / n) : 0u; };
+    for (int s = 0, Ns = 1; s < k; Ns *= a.radix[s], ++s) {
+        a.step[s] = L / (Ns * a.radix[s]);
+        a.mg[s] = magic(Ns);
+    }
+    a.mgL = magic(L);
+    a.mgW = magic(L / 2 + 1);
     return a;
 }
 

@@ -19,10 +19,15 @@ constexpr int kNumKernels = 5;     // per species: shell, ball, vector shell x, 
 constexpr int kMaxStages = 16;
 
 // Mixed-radix (4, 2, 3, 5) Stockham plan of one axis.
+// mg* are 32-bit reciprocals ceil(2^32 / n) for division by multiply-high (0 for
+// n = 1), exact while numerator x n < 2^32.
 struct FftAxis {
     int L;
     int nst;
     int radix[kMaxStages];
+    int step[kMaxStages];          // L / (Ns radix), Ns the product of the earlier radices
+    unsigned mg[kMaxStages];       // division by Ns
+    unsigned mgL, mgW;             // by L and by L / 2 + 1
 };
 
 bool smooth235(int n);
