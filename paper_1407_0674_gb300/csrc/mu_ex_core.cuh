@@ -778,8 +778,8 @@ template <auto K> static void ensure_smem() {
 constexpr long kSmemCap = 200 * 1024;
 constexpr int kMaxThreads = 256;
 
-// Threads per CTA of the x and y kernels and columns per CTA of the z kernels,
-// unless tuned.  A line's transform meets at four block barriers, so a CTA
+// Threads per CTA of the x kernels and columns per CTA of the y kernels, unless
+// tuned.  A line's transform meets at four block barriers, so a CTA
 // should be no larger than its loads need: with 256 threads the FP64 kernels
 // lose 10 to 30 % at the barriers, and double-float at 256 points, which fills
 // its registers, is the one kernel that prefers them.  Measured (us, 256
@@ -798,19 +798,64 @@ template <typename T> static int y_columns(int L) {
     if (std::is_same<T, float>::value) return 8;
     return L == 256 || L == 80 ? 16 : 8;
 }
-// one warp per z CTA at 128 points in FP32 and double-float: a 96^3 film's z MAC
-// and z back take 69 and 86 us for 84 and 113 (FP32), 302 and 291 us for 394 and
-// 386 (double-float)
-template <typename T> static int z_columns(int L, int fits) {
-    return L == 128 && !std::is_same<T, double>::value ? 1 : fits;
+// CTAs of a z kernel, and their waves with `occ` on an SM
+static long z_ctas(const Dims &d, int tx) { return (long)((d.Wx + tx - 1) / tx) * (d.Ly / 2 + 1); }
+static long z_waves(const Dims &d, int tx, int occ) { return (z_ctas(d, tx) + 152L * occ - 1) / (152L * occ); }
+// At 128 points a z kernel's CTAs take one to three waves on common grids, so the
+// fewest waves decide the columns per CTA and, in FP64, the CTAs per SM (by the
+// shared memory `sm` asked for).
+// FP32, double-float: a 96^3 film's z MAC and z back take 302 and 291 us in one
+// wave of one-warp CTAs, 394 and 386 in two waves of larger ones (FP32 69 and 86
+// for 84 and 113); a 100^3 film has two waves either way and keeps the larger.
+// FP64 waits for its pipe: two columns (100^3: 690 us; 950 at one, 697 at four),
+// and a wave of three CTAs an SM takes 213 us where one of four takes 235, so
+// three if they need no more waves and fill them to 7/8: z MAC 679 -> 636 us at
+// 96^3, 689 -> 644 at 100^3, but 241 -> 407 at 64, 923 -> 1041 at 120 (more waves)
+// and 5 % more on 693 CTAs (1.5 waves), which stay at four.
+template <typename T, typename K>
+static int z_columns(K kernel, int G, long per_col, size_t table, const Dims &d, int fits, size_t *sm) {
+    *sm = 0;
+    if (d.Lz != 128) return fits;
+    int best = std::is_same<T, double>::value ? std::min(fits, 2) : fits;
+    long least = 0;
+    for (int tx = best; tx >= 1; tx /= 2) {
+        int occ = 0;
+        const size_t need = 2 * tx * per_col + table;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 2 * tx * G, need) != cudaSuccess || occ < 1)
+            continue;
+        const long waves = z_waves(d, tx, occ);
+        if (std::is_same<T, double>::value) {
+            if (occ == 4 && z_waves(d, tx, 3) == waves && z_ctas(d, tx) * 8 >= 152 * 3 * waves * 7) *sm = 228 * 1024 / 4;
+            return tx;
+        }
+        if (!least || waves < least) {
+            least = waves;
+            best = tx;
+        }
+    }
+    return best;
 }
 
 // lines per CTA of the x kernels: the tuned tile if set, else x_threads; at most
-// kMaxThreads threads, the shared-memory cap and the line pairs there are
+// kMaxThreads threads, the shared-memory cap and the line pairs there are.  Not
+// tuned, the largest such number that gives a plane the fewest warps: 20 line
+// pairs of 40 points in CTAs of 16 ran 8 warps for 5, an x stage of 56 us against
+// 51 with one CTA (40 x 40 x 100, double-float)
 template <typename T> static int x_lines(const Problem *p, int L, int G, long ex_bytes, int npairs) {
     int P = p->tile[0] > 0 ? p->tile[0] : std::max(1, x_threads<T>(L) / G);
     P = std::min<long>(P, std::min<long>(kMaxThreads / G, kSmemCap / ex_bytes));
-    return std::max(1, std::min(P, npairs));
+    P = std::max(1, std::min(P, npairs));
+    if (p->tile[0] > 0) return P;
+    int best = P;
+    long least = 0;
+    for (; P >= 1; --P) {
+        const long warps = (long)((npairs + P - 1) / P) * ((P * G + 31) / 32);
+        if (!least || warps < least) {
+            least = warps;
+            best = P;
+        }
+    }
+    return best;
 }
 
 // split derivative stage (see stage 5 of run_pipeline)
@@ -889,8 +934,11 @@ static bool launch_zreg(bool back, int s, bool msa, typename vec2<T>::type *B10,
 
 // z kernels in the wide form where the paired-column form's warps would not
 // give every quarter of an SM one (kWideWarps); false otherwise.  The MSA term
-// stays with the paired-column kernel.
-constexpr long kWideWarps = 4 * 152;
+// stays with the paired-column kernel.  The z MAC at lengths whose columns take a
+// warp each (48, 80, 96), and in FP64, needs a second wave of its larger CTAs
+// above three warps per SM (kWideMacWarps): 173 us wide against 184 on 325 FP64
+// columns of 80 points, 236 against 197 on 481; the z back is 173 against 196 there.
+constexpr long kWideWarps = 4 * 152, kWideMacWarps = 3 * 152;
 template <typename T, int N1, int N2>
 static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>::type *B10,
                          typename vec2<T>::type *Bs, const Dims &d, const typename vec2<T>::type *twz, const T *spec,
@@ -899,7 +947,8 @@ static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>
         return false;
     } else {
         constexpr int G = Shape<N1, N2>::G;
-        if (plain_warps >= kWideWarps || (back && msa) || sc.s > kWideGroups) return false;
+        const bool short_mac = !back && (G > 8 || std::is_same<T, double>::value);
+        if (plain_warps >= (short_mac ? kWideMacWarps : kWideWarps) || (back && msa) || sc.s > kWideGroups) return false;
         int TX = 1;
         while (TX < 4 && 4 * TX * G * kWideGroups <= kWideThreads &&
                wide_smem<T, N1, N2>(back, sc.s, 2 * TX) <= (size_t)96 * 1024)
@@ -1011,14 +1060,22 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
                 // slots (with N1 lanes' worth of them, L = 80 ran 8 warps per SM)
                 const long per_col = ((long)s * N1 * N2 + Shape<N1, N2>::EX) * (long)cs;
                 int TX = pow2_le(std::max<long>(1, std::min<long>(std::min<long>(128 / G, 8), kBudget / (2 * per_col))));
-                TX = z_columns<T>(d.Lz, TX);
+                size_t few;
+                if (back) {
+                    ensure_smem<k_zback_p<T, N1, N2>>();
+                    TX = z_columns<T>(k_zback_p<T, N1, N2>, G, per_col, (size_t)G * G * cs, d, TX, &few);
+                } else {
+                    ensure_smem<k_zmac_p<T, N1, N2>>();
+                    TX = z_columns<T>(k_zmac_p<T, N1, N2>, G, per_col, (size_t)G * G * cs, d, TX, &few);
+                }
                 while (TX > 1 && (long)((d.Wx + TX - 1) / TX) * (d.Ly / 2 + 1) < 2 * 152) TX /= 2;
                 if (p->tile[2] > 0)
                     TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
                                                                                     (kSmemCap - (long)G * G * cs) /
                                                                                         (2 * per_col))));
                 dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
-                const size_t sm = 2 * TX * per_col + (size_t)G * G * cs;   // + twiddle table
+                size_t sm = 2 * TX * per_col + (size_t)G * G * cs;   // + twiddle table
+                if (p->tile[2] <= 0) sm = std::max(sm, few);
                 if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)g.x * g.y * ((2 * TX * G + 31) / 32), B10, Bs, d, twz,
                                             spec, sc, st))
                     return;

@@ -355,6 +355,13 @@ __device__ __forceinline__ void load_spec(T (&g)[kChunk][N1], const T *__restric
     }
 }
 
+// Zero-extended columns of at most half the length skip the zero butterflies in
+// the 64-bit paired-column kernels; in FP32 the second form of the stage costs
+// more than it saves (z MAC of 48 points on 64 x 64 columns 33 -> 39 us).
+template <typename T, int L> __device__ __forceinline__ bool half_column(int nz) {
+    return !std::is_same<T, float>::value && 2 * nz <= L;
+}
+
 template <typename T, int N1, int N2>
 __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__restrict__ Bs,
                                                  typename vec2<T>::type *__restrict__ B10, Dims d,
@@ -397,7 +404,7 @@ __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__
                 v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
             }
         }
-        fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
+        fwd2<N1, N2>(v, lt, ex, t, lanes, half_column<T, N1 * N2>(d.nz));
         if (t < N2) {
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) slot(i, k1) = v[k1];
@@ -436,7 +443,7 @@ __global__ void __launch_bounds__(256) k_zmac_p(const typename vec2<T>::type *__
                     }
                 }
             }
-            inv2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
+            inv2<N1, N2>(v, lt, ex, t, lanes, half_column<T, N1 * N2>(d.nz));
             if (t < N1 && ok) {
                 C *dst = B10 + (size_t)alpha * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
@@ -499,7 +506,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
                     v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
                 }
             }
-            fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
+            fwd2<N1, N2>(v, lt, ex, t, lanes, half_column<T, N1 * N2>(d.nz));
             if (t < N2) {
                 for (int i0 = 0; i0 < sc.s; i0 += kChunk) {
                     if (o == 0 || sc.s > kChunk) load_spec<T, N1, N2>(g, spec, d, sc.s, i0, type, kx, ky, t, ok);
@@ -542,7 +549,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
                     v[n2] = (ok && zz < d.nz) ? src[(size_t)zz * plane] : C{0, 0};
                 }
             }
-            fwd2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
+            fwd2<N1, N2>(v, lt, ex, t, lanes, half_column<T, N1 * N2>(d.nz));
             if (t < N2) {
                 for (int i = 0; i < sc.s; ++i) {
                     const T *base = spec + (size_t)(sc.s * kNumKernels + msa_pair(i, j, sc.s)) * oct +
@@ -565,7 +572,7 @@ __global__ void __launch_bounds__(256) k_zback_p(const typename vec2<T>::type *_
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) v[k1] = slot(i, k1);
         }
-        inv2<N1, N2>(v, lt, ex, t, lanes, 2 * d.nz <= N1 * N2);
+        inv2<N1, N2>(v, lt, ex, t, lanes, half_column<T, N1 * N2>(d.nz));
         if (t < N1 && ok) {
             C *dst = Bs + (size_t)i * d.nz * plane + (size_t)ky * d.Wx + kx;
 #pragma unroll
@@ -869,7 +876,7 @@ __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__
     const size_t plane = (size_t)d.Ly * d.Wx;
     const C *col = B10 + (size_t)ky * d.Wx + kx;
     C nxt[H];
-    zreg_load<N1, H>(nxt, col, ok, t, d.nz, plane);
+    if constexpr (HALF) zreg_load<N1, H>(nxt, col, ok, t, d.nz, plane);
     stage_type_spectra(specS, spec, d, S, 0, fy, kx0, TX);
     SmemTw<N1, N2, C>::fill(twtab, tw);
     __syncthreads();
@@ -888,10 +895,16 @@ __global__ void __launch_bounds__(128, 2) k_zback_reg(const float2 *__restrict__
         wide_entry(e + 1, type1, alpha1);
         const bool first = e == 0 || e == 3 || e == 4 || e == 6 || e == 8;
         const bool flip_y = type == 3 && ky > d.Ly / 2;
+        if constexpr (HALF) {
 #pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) v[n2] = n2 < H ? nxt[n2 < H ? n2 : 0] : C{0, 0};
-        if (e + 1 < kNumWeighted)
-            zreg_load<N1, H>(nxt, col + (size_t)alpha1 * d.nz * plane, ok, t, d.nz, plane);
+            for (int n2 = 0; n2 < N2; ++n2) v[n2] = n2 < H ? nxt[n2 < H ? n2 : 0] : C{0, 0};
+            if (e + 1 < kNumWeighted)
+                zreg_load<N1, H>(nxt, col + (size_t)alpha1 * d.nz * plane, ok, t, d.nz, plane);
+        } else {
+            // 16 rows ahead do not fit the registers beside the accumulators
+            // (0.567 -> 0.610 ms at 200 rows)
+            zreg_load<N1, H>(v, col + (size_t)alpha * d.nz * plane, ok, t, d.nz, plane);
+        }
         if (first) cp_async_wait_all_groups();
         fwd2<N1, N2>(v, lt, ex, t, lanes, HALF);
         if (first && type + 1 < kNumKernels)
