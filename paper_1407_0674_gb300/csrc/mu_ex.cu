@@ -479,7 +479,18 @@ static void free_mu_graph(MuGraph *m) {
     delete m;
 }
 
+// Creating the stream and the executable graph are among the calls that CUDA
+// forbids while any stream of the program is being captured in the default mode
+// (they invalidate that capture); recording has nothing to do with it, so it
+// runs in the relaxed mode.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 static bool record_mu_graph(Problem *p, int prec, const double *d_rho, double *d_mu, MuGraph *m) {
+    RelaxedCapture relaxed;
     cudaStream_t cap = nullptr;
     if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return false;
     bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed) == cudaSuccess;

@@ -88,3 +88,28 @@ def test_wide_z_kernels_match_oracle(pnp, length, species):
         for precision in ("fp64", "df64"):
             mu = P.excess_mu(rho, precision=precision)
             assert np.abs(mu - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+def test_small_calls_beside_a_capture(pnp, mode):
+    """Calls on one stream, the one that records the graph among them, leave a
+    capture under way on another stream intact."""
+    import torch
+    spec, rho = mu_microbench(12)
+    d = torch.from_numpy(rho).cuda()
+    with pnp.Problem(spec) as P:
+        want = torch.empty_like(d)
+        P.excess_mu_device(d, want)               # buffers and spectra exist from here on
+        assert P.status() == pnp.OK
+        outs = [torch.full_like(d, np.nan) for _ in range(4)]
+        x, side = torch.zeros(1000, device="cuda"), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, capture_error_mode=mode):
+            x += 1
+            for out in outs:
+                P.excess_mu_device(d, out, stream=side.cuda_stream)
+        g.replay()
+        torch.cuda.synchronize()
+        assert float(x[0]) == 1.0 and P.status() == pnp.OK
+        assert all(torch.equal(out, want) for out in outs)
