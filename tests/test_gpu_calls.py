@@ -113,3 +113,32 @@ def test_small_calls_beside_a_capture(pnp, mode):
         torch.cuda.synchronize()
         assert float(x[0]) == 1.0 and P.status() == pnp.OK
         assert all(torch.equal(out, want) for out in outs)
+
+
+def test_small_calls_keep_their_stream_priority(pnp):
+    """Calls on a high-priority stream finish while a kernel of many more blocks
+    than the GPU holds is still running on another stream; at equal priority they would
+    wait for its last block.  The last call is on a stream of the default priority,
+    after which the first stream's calls are still ahead."""
+    import torch
+    spec, rho = mu_microbench(12)
+    d = torch.from_numpy(rho).cuda()
+    big = torch.full((400_000_000,), 0.3, dtype=torch.float64, device="cuda")
+    torch.sin_(big)                               # 13 ms of FP64 arithmetic, no library start-up below
+    hi, low, work = torch.cuda.Stream(priority=-1), torch.cuda.Stream(), torch.cuda.Stream()
+    with pnp.Problem(spec) as P:
+        want, out = torch.empty_like(d), torch.empty_like(d)
+        P.excess_mu_device(d, want)
+        assert P.status() == pnp.OK
+        for call, stream in enumerate([hi] * 6 + [low, hi, hi]):
+            out.fill_(np.nan)
+            torch.cuda.synchronize()
+            done = torch.cuda.Event()
+            with torch.cuda.stream(work):
+                torch.sin_(big)
+                done.record(work)
+            P.excess_mu_device(d, out, stream=stream.cuda_stream)
+            stream.synchronize()
+            assert stream is low or not done.query(), call
+            torch.cuda.synchronize()
+            assert torch.equal(out, want)
