@@ -491,11 +491,14 @@ struct RelaxedCapture {
 
 static bool record_mu_graph(Problem *p, int prec, const double *d_rho, double *d_mu, MuGraph *m) {
     RelaxedCapture relaxed;
+    MuEnds ends;
     cudaStream_t cap = nullptr;
     if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return false;
     bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed) == cudaSuccess;
     if (ok) {
+        p->ends = &ends;
         ok = mu_ex_enqueue(p, prec, d_rho, d_mu, cap) == PNP_OK;
+        p->ends = nullptr;
         ok = cudaStreamEndCapture(cap, &m->graph) == cudaSuccess && ok;
     }
     cudaStreamDestroy(cap);
@@ -510,11 +513,14 @@ static bool record_mu_graph(Problem *p, int prec, const double *d_rho, double *d
         ok = cudaGraphNodeGetDependentNodes(nodes[k], nullptr, nullptr, &deps) == cudaSuccess;
         if (ok && deps == 0) m->node[1] = nodes[k];
     }
-    const bool reg = with_shape(p->L[0], [](auto, auto) {});
-    const int count[2] = {reg ? 6 : 7, reg ? 9 : 10};   // arguments of k_xfwd_r or k_xfwd, k_xinv_r or k_xinv
+    // the ends are the kernels that run_pipeline launched there, with this
+    // call's pointers in the places that later calls set
+    const void *ptr[2] = {d_rho, d_mu};
     for (int k = 0; ok && k < 2; ++k) {
-        ok = m->node[k] && cudaGraphKernelNodeGetParams(m->node[k], &m->prm[k]) == cudaSuccess;
-        if (ok) m->args[k].assign(m->prm[k].kernelParams, m->prm[k].kernelParams + count[k]);
+        ok = m->node[k] && cudaGraphKernelNodeGetParams(m->node[k], &m->prm[k]) == cudaSuccess &&
+             m->prm[k].func == ends.fn[k] && m->prm[k].kernelParams && ends.args[k] > kPointerArg[k];
+        if (ok) ok = *(const void *const *)m->prm[k].kernelParams[kPointerArg[k]] == ptr[k];
+        if (ok) m->args[k].assign(m->prm[k].kernelParams, m->prm[k].kernelParams + ends.args[k]);
     }
     return ok && cudaGraphInstantiate(&m->exec, m->graph, 0) == cudaSuccess;
 }

@@ -970,6 +970,12 @@ static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>
     }
 }
 
+template <typename... A> static void note_end(const Problem *p, int k, void (*fn)(A...)) {
+    if (!p->ends) return;
+    p->ends->fn[k] = (const void *)fn;
+    p->ends->args[k] = (int)sizeof...(A);
+}
+
 template <typename T>
 static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, double *d_mu, cudaStream_t st,
                         bool tc = false) {
@@ -1001,9 +1007,11 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
             ensure_smem<k_xfwd_r<T, N1, N2>>();
             dim3 g((d.npairs + P - 1) / P, d.nz, s);
             k_xfwd_r<T, N1, N2><<<g, P * G, P * Shape<N1, N2>::EX * cs, st>>>(d_rho, N, A, d, twx, P);
+            note_end(p, 0, k_xfwd_r<T, N1, N2>);
         })) {
         dim3 gx((d.npairs + l.P_x - 1) / l.P_x, d.nz, s);
         k_xfwd<T><<<gx, T256, l.sm_x, st>>>(d_rho, N, A, d, p->ax[0], twx, l.P_x);
+        note_end(p, 0, k_xfwd<T>);
     }
     tm.end(st);
 
@@ -1162,9 +1170,11 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
             ensure_smem<k_xinv_r<T, N1, N2>>();
             dim3 g((d.npairs + P - 1) / P, d.nz, s);
             k_xinv_r<T, N1, N2><<<g, P * G, P * Shape<N1, N2>::EX * cs, st>>>(A, d_mu, N, d, twx, U, sc, P, E);
+            note_end(p, 1, k_xinv_r<T, N1, N2>);
         })) {
         dim3 gx((d.npairs + l.P_x - 1) / l.P_x, d.nz, s);
         k_xinv<T><<<gx, T256, l.sm_x, st>>>(A, d_mu, N, d, p->ax[0], twx, U, sc, l.P_x, E);
+        note_end(p, 1, k_xinv<T>);
     }
     tm.end(st);
     return cuda_status(cudaGetLastError());

@@ -68,6 +68,12 @@ struct StageTimer {
 };
 struct GummelState;     // device state of the Gummel solve
 struct MuGraph;         // one mu_ex call recorded as a graph (mu_ex.cu)
+// the kernels that read the densities and write the result of a mu_ex call, and
+// their numbers of arguments; filled by run_pipeline for a call being recorded
+struct MuEnds {
+    const void *fn[2] = {nullptr, nullptr};
+    int args[2] = {0, 0};
+};
 
 struct Problem {
     // ---- descriptor (copied) ----
@@ -123,6 +129,7 @@ struct Problem {
     int deferred = 0;                 // host-side deferred status
     StageTimer timer;
     MuGraph *mug[4] = {nullptr, nullptr, nullptr, nullptr};   // small grids: one call as a graph, per precision
+    MuEnds *ends = nullptr;           // set while one is recorded
     int mg_levels = 0;
     int tile[3] = {0, 0, 0};          // register-FFT CTA tiles (x lines, y columns, z columns); 0: rule
     double tuned_ms = 0;              // mu_ex time measured by the autotuner

@@ -118,8 +118,8 @@ def test_small_calls_beside_a_capture(pnp, mode):
 def test_small_calls_keep_their_stream_priority(pnp):
     """Calls on a high-priority stream finish while a kernel of many more blocks
     than the GPU holds is still running on another stream; at equal priority they would
-    wait for its last block.  The last call is on a stream of the default priority,
-    after which the first stream's calls are still ahead."""
+    wait for its last block.  One call is on a stream of the default priority; those
+    after it, on the first stream again, are still ahead."""
     import torch
     spec, rho = mu_microbench(12)
     d = torch.from_numpy(rho).cuda()
@@ -142,3 +142,33 @@ def test_small_calls_keep_their_stream_priority(pnp):
             assert stream is low or not done.query(), call
             torch.cuda.synchronize()
             assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("case,precision", [("wells", "fp64"), ("wells", "df64"), ("msa", "fp64"), ("msa", "fp32"),
+                                            ("white bear", "fp64"), ("y 256", "tf32split")])
+def test_graph_calls_of_every_option(pnp, case, precision):
+    """The recorded graph takes each call's own buffers with every part of the pipeline on."""
+    import torch
+    from workloads import film_gummel, lognormal_density
+    if case == "wells":
+        spec = film_gummel(12, 10, 14, nsites=4)
+        rho = lognormal_density(spec, 5, sigma=0.2)
+    else:
+        spec, rho = mu_microbench(shape=(12, 100, 9) if case == "y 256" else (12, 10, 9))
+        spec.msa, spec.fmt = case == "msa", int(case == "white bear")
+        if case == "y 256":
+            spec.fft_len = (16, 256, 16)          # the length that the tensor-core y pass takes
+    ins = [torch.from_numpy(rho * f).cuda() for f in (1.0, 0.5, 0.9)]
+    with pnp.Problem(spec, precision=precision) as P:
+        outs = [torch.full_like(ins[0], np.nan) for _ in range(7)]
+        torch.cuda.synchronize()
+        for k, out in enumerate(outs):
+            P.excess_mu_device(ins[k % 3], out)
+            assert P.status() == pnp.OK
+        P.stage_timing(True)                      # timed calls are launched one by one
+        for k, out in enumerate(outs):
+            want = torch.full_like(out, np.nan)
+            torch.cuda.synchronize()
+            P.excess_mu_device(ins[k % 3], want)
+            assert P.status() == pnp.OK
+            assert torch.equal(out, want), k
