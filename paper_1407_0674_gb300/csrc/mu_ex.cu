@@ -547,14 +547,17 @@ int mu_ex_launch(Problem *p, int prec, const double *d_rho, double *d_mu, cudaSt
     }
     NvtxRange range("mu_ex");
     const void *ptr[2] = {d_rho, d_mu};
-    for (int k = 0; k < 2; ++k) {
+    bool ok = true;
+    for (int k = 0; ok && k < 2; ++k) {
         cudaKernelNodeParams prm = m->prm[k];
         m->args[k][kPointerArg[k]] = &ptr[k];
         prm.kernelParams = m->args[k].data();
-        const cudaError_t e = cudaGraphExecKernelNodeSetParams(m->exec, m->node[k], &prm);
-        if (e != cudaSuccess) return cuda_status(e);
+        ok = cudaGraphExecKernelNodeSetParams(m->exec, m->node[k], &prm) == cudaSuccess;
     }
-    return cuda_status(cudaGraphLaunch(m->exec, st));
+    if (ok && cudaGraphLaunch(m->exec, st) == cudaSuccess) return PNP_OK;
+    cudaGetLastError();
+    m->failed = true;                          // launches from here on, with their own errors
+    return mu_ex_enqueue(p, prec, d_rho, d_mu, st);
 }
 
 // ---------------------------------------------------------------------------
