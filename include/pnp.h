@@ -248,12 +248,20 @@ int pnp_plan_problem(const pnp_problem_desc *desc, pnp_problem_info *info, doubl
  * the Rosenfeld derivatives dPhi/dn_alpha in FP64, masked to the domain, and
  * their back-convolution (Sec 2.3.1, Sec 3.4); plus the cached square-well
  * term (Sec 2.3.2).  Writes mu_ex [s][nz][ny][nx] (host).  Blocks until done.
- * Errors: PNP_ERR_INVALID, PNP_ERR_PACKING (n3 >= 1 somewhere), PNP_ERR_CUDA. */
+ * The densities are checked on the device: negative or non-finite ones are
+ * refused (PNP_ERR_INVALID) with mu_ex and a status pending from earlier device
+ * calls left as they were, but a call of fewer than 2^22 values may have taken
+ * the time of a full one by then.
+ * Errors: PNP_ERR_INVALID, PNP_ERR_PACKING (n3 >= 1 somewhere), PNP_ERR_NOMEM,
+ * PNP_ERR_CUDA. */
 int pnp_excess_mu(pnp_problem *p, const double *rho, double *mu_ex, int precision);
 
 /* As pnp_excess_mu with device pointers, enqueued on `stream` (a
  * cudaStream_t, NULL = the problem's stream).  Does not synchronise; a
- * packing error is reported by the next pnp_status(). */
+ * packing error is reported by the next pnp_status().  On small grids (species x
+ * points at most 400000) the third call of a precision records the call's
+ * kernels as a CUDA graph, which later calls launch with their own pointers; a
+ * stream under capture gets the kernels themselves. */
 int pnp_excess_mu_device(pnp_problem *p, const double *d_rho, double *d_mu_ex, int precision,
                          void *stream);
 

@@ -137,8 +137,8 @@ int create_problem_internal(const pnp_problem_desc *desc, Problem **out, std::st
     }
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = dmalloc((void **)&p->d_flag, sizeof(int), p->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_flag, 0, sizeof(int), p->stream);
+    if (e == cudaSuccess) e = dmalloc((void **)&p->d_flag, kFlagWords * sizeof(int), p->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_flag, 0, kFlagWords * sizeof(int), p->stream);
     if (e != cudaSuccess) {
         rc = cuda_status(e);
         destroy_problem_internal(p);
@@ -155,6 +155,13 @@ int create_problem_internal(const pnp_problem_desc *desc, Problem **out, std::st
     return PNP_OK;
 }
 
+static int status_of(int h) {
+    if (h & kFlagTimeout) return PNP_ERR_TIMEOUT;
+    if (h & kFlagOverflow) return PNP_ERR_OVERFLOW;
+    if (h & (kFlagPacking | kFlagNonFinite)) return PNP_ERR_PACKING;
+    return PNP_OK;
+}
+
 static int read_flag(Problem *p, cudaStream_t st) {
     int h = 0;
     cudaError_t e = cudaMemcpyAsync(&h, p->d_flag, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -164,11 +171,35 @@ static int read_flag(Problem *p, cudaStream_t st) {
         cudaMemsetAsync(p->d_flag, 0, sizeof(int), st);
         cudaStreamSynchronize(st);
     }
-    if (h & kFlagInvalid) return PNP_ERR_INVALID;
-    if (h & kFlagTimeout) return PNP_ERR_TIMEOUT;
-    if (h & kFlagOverflow) return PNP_ERR_OVERFLOW;
-    if (h & (kFlagPacking | kFlagNonFinite)) return PNP_ERR_PACKING;
-    return PNP_OK;
+    return status_of(h);
+}
+
+// The verdict of check_values_enqueue, once the stream has got there.
+static int read_refusal(Problem *p, cudaStream_t st) {
+    int h = 0;
+    cudaError_t e = cudaMemcpyAsync(&h, p->d_flag + kWordRefused, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_status(e);
+    if (!h) return PNP_OK;
+    cudaMemsetAsync(p->d_flag + kWordRefused, 0, sizeof(int), st);
+    cudaStreamSynchronize(st);
+    return PNP_ERR_INVALID;
+}
+
+// Verdict and status of a host call's work.  Where its densities were refused the
+// status of earlier calls is pending as before.
+static int read_call(Problem *p, cudaStream_t st) {
+    int h[kFlagWords] = {0};
+    cudaError_t e = cudaMemcpyAsync(h, p->d_flag, sizeof(h), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_status(e);
+    const bool refused = h[kWordRefused];
+    if (refused || h[kWordStatus]) {
+        const int next[kFlagWords] = {refused ? h[kWordHeld] : 0, 0, 0};
+        cudaMemcpyAsync(p->d_flag, next, sizeof(next), cudaMemcpyHostToDevice, st);
+        cudaStreamSynchronize(st);
+    }
+    return refused ? (int)PNP_ERR_INVALID : status_of(h[kWordStatus]);
 }
 
 static int resolve_prec(const Problem *p, int prec) {
@@ -335,29 +366,45 @@ int pnp_excess_mu(pnp_problem *h, const double *rho, double *mu_ex, int precisio
     int prec = resolve_prec(p, precision);
     if (prec < 0) return PNP_ERR_INVALID;
     const size_t n = p->npts() * p->s;
+    // an error of the library's own is reported only for densities it would take
+    auto fail = [&](int rc) { return host_values_ok(rho, n, 1) ? rc : (int)PNP_ERR_INVALID; };
     if (!p->d_io) {
         if (dmalloc((void **)&p->d_io, sizeof(double) * (2 * n + p->npts()), p->stream) != cudaSuccess)
-            return PNP_ERR_NOMEM;
+            return fail(PNP_ERR_NOMEM);
         p->device_bytes += sizeof(double) * (2 * n + p->npts());
     }
-    cudaStream_t st = p->stream;
-    p->last_stream = st;
     // The densities are checked on the device, and the pages of a fresh output
     // array are touched while it computes: the host's scan and the page faults
     // of the copy back were 0.55 and 0.40 of the 0.86 ms of a 64^3 FP32 call.
-    // Nothing is copied back for densities that fail the check.
+    // Nothing is copied back for densities that fail the check.  mu_ex starts
+    // without waiting for the verdict (waiting: 64^3 343 -> 364 us, 32^3 95 ->
+    // 111), except where a refusal would have spent much more on it than the wait
+    // (kCheckFirst values: calls of 1.2 ms and more), or where a device call on
+    // another stream may be at work in the workspace, which only a call that is
+    // taken may disturb.
+    constexpr size_t kCheckFirst = (size_t)1 << 22;
+    cudaStream_t st = p->stream;
     cudaError_t e = cudaMemcpyAsync(p->d_io, rho, sizeof(double) * n, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_flag, 0, sizeof(int), st);
-    if (e != cudaSuccess) return cuda_status(e);
-    int rc = check_values_enqueue(p, p->d_io, n, st);
-    if (rc == PNP_OK) rc = mu_ex_launch(p, prec, p->d_io, p->d_io + n, st);
+    if (e != cudaSuccess) return fail(cuda_status(e));
+    const bool wait = n >= kCheckFirst || p->last_stream != st;
+    int rc = check_values_enqueue(p, p->d_io, n, !wait, st);
+    if (rc) return fail(rc);
+    if (wait) {
+        rc = read_refusal(p, st);
+        if (rc == PNP_OK) rc = cuda_status(cudaMemsetAsync(p->d_flag, 0, kFlagWords * sizeof(int), st));
+        if (rc) return rc;
+    }
+    rc = mu_ex_launch(p, prec, p->d_io, p->d_io + n, st);
+    if (rc == PNP_OK) touch_pages(mu_ex, sizeof(double) * n);
+    const int status = read_call(p, st);
+    if (status == PNP_ERR_INVALID) return status;
+    p->last_stream = st;
     if (rc) return rc;
-    touch_pages(mu_ex, sizeof(double) * n);
-    rc = read_flag(p, st);
-    if (rc != PNP_OK && rc != PNP_ERR_PACKING && rc != PNP_ERR_OVERFLOW && rc != PNP_ERR_TIMEOUT) return rc;
+    if (status != PNP_OK && status != PNP_ERR_PACKING && status != PNP_ERR_OVERFLOW && status != PNP_ERR_TIMEOUT)
+        return status;
     e = cudaMemcpyAsync(mu_ex, p->d_io + n, sizeof(double) * n, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return e == cudaSuccess ? rc : cuda_status(e);
+    return e == cudaSuccess ? status : cuda_status(e);
 }
 
 int pnp_excess_mu_device(pnp_problem *h, const double *d_rho, double *d_mu_ex, int precision, void *stream) {

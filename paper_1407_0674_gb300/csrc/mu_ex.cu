@@ -438,15 +438,21 @@ int mu_ex_enqueue(Problem *p, int prec, const double *d_rho, double *d_mu, cudaS
 
 // The check of a host call's densities, on the device copy: the host's scan of
 // 64^3 x 3 values took 0.55 ms of a 0.86 ms call, this 3 us.
-static __global__ void k_check_values(const double *__restrict__ x, size_t n, int *__restrict__ flag) {
+// With `hold` the status is cleared too, the one pending from earlier calls kept
+// for a refusal.
+static __global__ void k_check_values(const double *__restrict__ x, size_t n, int *__restrict__ flag, bool hold) {
     bool ok = true;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         ok = ok && x[i] >= 0.0 && isfinite(x[i]);
-    if (!ok) atomicOr(flag, kFlagInvalid);
+    if (!ok) flag[kWordRefused] = 1;
+    if (hold && blockIdx.x == 0 && threadIdx.x == 0) {
+        flag[kWordHeld] = flag[kWordStatus];
+        flag[kWordStatus] = 0;
+    }
 }
 
-int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st) {
-    k_check_values<<<(int)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(d, n, p->d_flag);
+int check_values_enqueue(Problem *p, const double *d, size_t n, bool hold, cudaStream_t st) {
+    k_check_values<<<(int)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(d, n, p->d_flag, hold);
     return cuda_status(cudaGetLastError());
 }
 

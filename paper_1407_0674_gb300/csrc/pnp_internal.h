@@ -115,7 +115,7 @@ struct Problem {
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t last_stream = nullptr;
-    int *d_flag = nullptr;            // device status bits
+    int *d_flag = nullptr;            // device status bits (kWordStatus), then the words of a host call's check
     double *d_U = nullptr;            // square-well field sum_m K_sw[m] rho_s(r+m)
     std::vector<double> sh_coef;      // mu_sh,i = sh_coef[i] * U
     double *d_E = nullptr;            // [s][N] MSA bulk field sum_j rho_b,j (C_ij (x) 1_Omega)
@@ -170,8 +170,8 @@ int mu_ex_prepare(Problem *p, int prec);     // lazily build one precision's buf
 int mu_ex_enqueue(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st);
 int mu_ex_launch(Problem *p, int prec, const double *d_rho, double *d_mu, cudaStream_t st);   // one call's work
 void mu_ex_free(Problem *p);
-// sets kFlagInvalid in p->d_flag unless every d[k] is finite and >= 0
-int check_values_enqueue(Problem *p, const double *d, size_t n, cudaStream_t st);
+// sets kWordRefused unless every d[k] is finite and >= 0; `hold`: the status moves to kWordHeld
+int check_values_enqueue(Problem *p, const double *d, size_t n, bool hold, cudaStream_t st);
 // F_sh (Sec 2.3.2) of device densities into d_out[0] (d_part: 512 doubles)
 int square_well_energy_enqueue(Problem *p, const double *d_rho, double *d_out, double *d_part, cudaStream_t st);
 
@@ -205,7 +205,9 @@ int create_problem_internal(const pnp_problem_desc *desc, Problem **out, std::st
 void destroy_problem_internal(Problem *p);
 
 // device status bits
-enum : int { kFlagPacking = 1, kFlagOverflow = 2, kFlagNonFinite = 4, kFlagTimeout = 8, kFlagInvalid = 16 };
+enum : int { kFlagPacking = 1, kFlagOverflow = 2, kFlagNonFinite = 4, kFlagTimeout = 8 };
+// words of d_flag: the status bits, a refused host call's mark, the status before that call
+enum : int { kWordStatus = 0, kWordRefused = 1, kWordHeld = 2, kFlagWords = 3 };
 
 }  // namespace pnp
 

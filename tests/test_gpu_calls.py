@@ -172,3 +172,35 @@ def test_graph_calls_of_every_option(pnp, case, precision):
             P.excess_mu_device(ins[k % 3], want)
             assert P.status() == pnp.OK
             assert torch.equal(out, want), k
+
+
+@pytest.mark.parametrize("shape", [(10, 10, 10), (112, 112, 112)])    # before and after the check's verdict
+def test_refused_host_call_changes_nothing(pnp, shape):
+    """Refused densities leave a pending device status, the output and the next result as
+    they were, and are refused for what they are when memory runs out too."""
+    import torch
+    spec, rho = mu_microbench(shape=shape)
+    bad = rho.copy()
+    bad[2, -1, -1, -1] = -1.0
+    out = np.full_like(rho, 7.0)
+    with pnp.Problem(spec, precision="fp32") as P:
+        def refused():
+            rc = pnp.lib().pnp_excess_mu(P.h, pnp._ptr(bad), pnp._ptr(out), -1)
+            return rc == pnp.ERR_INVALID and (out == 7.0).all()
+        pnp.lib().pnp_test_fail_alloc_at(1)
+        try:
+            assert refused()
+        finally:
+            pnp.lib().pnp_test_fail_alloc_at(0)
+        d = torch.from_numpy(rho).cuda()
+        d_mu, packed = torch.empty_like(d), 4.0 * d
+        side = torch.cuda.Stream()
+        for stream in (None, side.cuda_stream):
+            torch.cuda.synchronize()
+            P.excess_mu_device(packed, d_mu, stream=stream)      # n3 above 1
+            torch.cuda.synchronize()
+            assert refused() and P.status() == pnp.ERR_PACKING
+            assert refused() and P.status() == pnp.OK
+        P.excess_mu_device(d, d_mu)
+        assert P.status() == pnp.OK
+        assert np.array_equal(P.excess_mu(rho), d_mu.cpu().numpy())
