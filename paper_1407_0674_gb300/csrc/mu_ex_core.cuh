@@ -801,6 +801,25 @@ template <typename T> static int y_columns(int L) {
 // CTAs of a z kernel, and their waves with `occ` on an SM
 static long z_ctas(const Dims &d, int tx) { return (long)((d.Wx + tx - 1) / tx) * (d.Ly / 2 + 1); }
 static long z_waves(const Dims &d, int tx, int occ) { return (z_ctas(d, tx) + 152L * occ - 1) / (152L * occ); }
+// Fewer columns per CTA where there would be less than two CTAs an SM, with two
+// limits.  CTAs of 8-lane columns have at most four warps, so splitting them only
+// helps where the fullest SM then holds fewer: 40 rows on 90 x 90 columns in FP64 148
+// us in 276 CTAs of four warps, 177 in 552 of two; but 64 rows on 64 x 64 195 us in
+// 165, 115 in 297.  And rows of a tile stay a 32-byte sector (48 rows on 64 x 64 in
+// FP32, z MAC and z back, 34 and 33 us with four columns, 39 and 35 with two; 80
+// rows on 32 x 64 in FP64 187 us with two, 200 with one), unless the fullest SM's
+// warps halve (80 rows on 32 x 64 in FP32 28.6 us with four, 27.4 with two).
+static int z_spread(const Dims &d, int tx, int G, size_t cs) {
+    auto fullest = [&](int t) { return z_waves(d, t, 1) * ((2 * t * G + 31) / 32); };
+    while (tx > 1 && z_ctas(d, tx) < 2 * 152) {
+        const long now = fullest(tx), next = fullest(tx / 2);
+        const bool sector = tx / 2 * cs >= 32;
+        if (sector ? G <= 8 && next >= now : 2 * next > now) break;
+        tx /= 2;
+    }
+    return tx;
+}
+
 // At 128 points a z kernel's CTAs take one to three waves on common grids, so the
 // fewest waves decide the columns per CTA and, in FP64, the CTAs per SM (by the
 // shared memory `sm` asked for).
@@ -935,15 +954,15 @@ static bool launch_zreg(bool back, int s, bool msa, typename vec2<T>::type *B10,
     }
 }
 
-// z kernels in the wide form where the paired-column form's warps would not
+// z kernels in the wide form where the columns' warps would not
 // give every quarter of an SM one (kWideWarps); false otherwise.  The MSA term
 // stays with the paired-column kernel.  The z MAC at lengths whose columns take a
 // warp each (48, 80, 96), and in FP64, needs a second wave of its larger CTAs
-// above three warps per SM (kWideMacWarps): 173 us wide against 184 on 325 FP64
-// columns of 80 points, 236 against 197 on 481; the z back is 173 against 196 there.
+// above three warps per SM (kWideMacWarps): 174 us wide against 184 on 325 FP64
+// columns of 80 points, 236 against 187 on 481; the z back is 172 against 184 there.
 constexpr long kWideWarps = 4 * 152, kWideMacWarps = 3 * 152;
 template <typename T, int N1, int N2>
-static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>::type *B10,
+static bool launch_zwide(bool back, bool msa, long warps, typename vec2<T>::type *B10,
                          typename vec2<T>::type *Bs, const Dims &d, const typename vec2<T>::type *twz, const T *spec,
                          const SpeciesConst &sc, cudaStream_t st) {
     if constexpr (N1 * N2 > kWideMaxLen) {
@@ -951,7 +970,7 @@ static bool launch_zwide(bool back, bool msa, long plain_warps, typename vec2<T>
     } else {
         constexpr int G = Shape<N1, N2>::G;
         const bool short_mac = !back && (G > 8 || std::is_same<T, double>::value);
-        if (plain_warps >= (short_mac ? kWideMacWarps : kWideWarps) || (back && msa) || sc.s > kWideGroups) return false;
+        if (warps >= (short_mac ? kWideMacWarps : kWideWarps) || (back && msa) || sc.s > kWideGroups) return false;
         int TX = 1;
         while (TX < 4 && 4 * TX * G * kWideGroups <= kWideThreads &&
                wide_smem<T, N1, N2>(back, sc.s, 2 * TX) <= (size_t)96 * 1024)
@@ -1079,7 +1098,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
                     ensure_smem<k_zmac_p<T, N1, N2>>();
                     TX = z_columns<T>(k_zmac_p<T, N1, N2>, G, per_col, (size_t)G * G * cs, d, TX, &few);
                 }
-                while (TX > 1 && (long)((d.Wx + TX - 1) / TX) * (d.Ly / 2 + 1) < 2 * 152) TX /= 2;
+                TX = z_spread(d, TX, G, cs);
                 if (p->tile[2] > 0)
                     TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
                                                                                     (kSmemCap - (long)G * G * cs) /
@@ -1087,7 +1106,7 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
                 dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
                 size_t sm = 2 * TX * per_col + (size_t)G * G * cs;   // + twiddle table
                 if (p->tile[2] <= 0) sm = std::max(sm, few);
-                if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)g.x * g.y * ((2 * TX * G + 31) / 32), B10, Bs, d, twz,
+                if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)d.Wx * (d.Ly / 2 + 1) * 2 * G / 32, B10, Bs, d, twz,
                                             spec, sc, st))
                     return;
                 if (back && sc.msa) {

@@ -54,3 +54,11 @@ def test_paired_column_kernels_match_oracle(pnp, length, species):
 def test_small_planes_in_fp32_match_oracle(pnp, length):
     check(pnp, (16, 16), length, 3, ("fp32",))
     check(pnp, (40, 24), length, 4, ("fp32",))
+
+
+# planes at the limits of the rule for the columns per CTA: rows of one sector, fewer
+# on planes whose fullest SM empties by half, few large CTAs of 8-lane columns
+@pytest.mark.parametrize("plane,length", [((64, 64), 48), ((40, 80), 48), ((32, 64), 80), ((32, 64), 96),
+                                          ((90, 90), 40), ((64, 64), 64), ((64, 64), 40), ((32, 64), 128)])
+def test_column_tiles_match_oracle(pnp, plane, length):
+    check(pnp, plane, length, 3, ("fp64", "df64", "fp32"))
