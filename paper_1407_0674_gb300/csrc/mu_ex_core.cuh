@@ -1085,39 +1085,41 @@ static int run_pipeline(Problem *p, DeviceBuffers *db, const double *d_rho, doub
         if (!with_shape(d.Lz, [&](auto a, auto b) {
                 constexpr int N1 = decltype(a)::value, N2 = decltype(b)::value, G = Shape<N1, N2>::G;
                 if (launch_zreg<T, N1, N2>(back, s, sc.msa != 0, B10, Bs, d, twz, spec, sc, st)) return;
+                if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)d.Wx * (d.Ly / 2 + 1) * 2 * G / 32, B10, Bs, d, twz,
+                                            spec, sc, st))
+                    return;
                 // paired columns (ky, Ly - ky): 2 TX columns per CTA
                 // a lane t < N2 keeps N1 values per species and column: N1 N2
                 // slots (with N1 lanes' worth of them, L = 80 ran 8 warps per SM)
                 const long per_col = ((long)s * N1 * N2 + Shape<N1, N2>::EX) * (long)cs;
-                int TX = pow2_le(std::max<long>(1, std::min<long>(std::min<long>(128 / G, 8), kBudget / (2 * per_col))));
-                size_t few;
-                if (back) {
-                    ensure_smem<k_zback_p<T, N1, N2>>();
-                    TX = z_columns<T>(k_zback_p<T, N1, N2>, G, per_col, (size_t)G * G * cs, d, TX, &few);
-                } else {
-                    ensure_smem<k_zmac_p<T, N1, N2>>();
-                    TX = z_columns<T>(k_zmac_p<T, N1, N2>, G, per_col, (size_t)G * G * cs, d, TX, &few);
-                }
-                TX = z_spread(d, TX, G, cs);
-                if (p->tile[2] > 0)
-                    TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
-                                                                                    (kSmemCap - (long)G * G * cs) /
-                                                                                        (2 * per_col))));
-                dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
-                size_t sm = 2 * TX * per_col + (size_t)G * G * cs;   // + twiddle table
-                if (p->tile[2] <= 0) sm = std::max(sm, few);
-                if (launch_zwide<T, N1, N2>(back, sc.msa != 0, (long)d.Wx * (d.Ly / 2 + 1) * 2 * G / 32, B10, Bs, d, twz,
-                                            spec, sc, st))
-                    return;
+                const size_t table = (size_t)G * G * cs;   // twiddles
+                auto go = [&](auto kernel, const C *in, C *out) {
+                    // the rule's tile, found once per problem (it asks for occupancies)
+                    ZRule &zt = p->ztile[prec][back];
+                    if (!zt.tx) {
+                        const int fits = pow2_le(
+                            std::max<long>(1, std::min<long>(std::min<long>(128 / G, 8), kBudget / (2 * per_col))));
+                        zt.tx = z_spread(d, z_columns<T>(kernel, G, per_col, table, d, fits, &zt.smem), G, cs);
+                    }
+                    int TX = zt.tx;
+                    if (p->tile[2] > 0)
+                        TX = std::max(1, std::min<int>(p->tile[2], (int)std::min<long>(kMaxThreads / (2 * G),
+                                                                                        (kSmemCap - (long)table) /
+                                                                                            (2 * per_col))));
+                    const dim3 g((d.Wx + TX - 1) / TX, d.Ly / 2 + 1);
+                    size_t sm = 2 * TX * per_col + table;
+                    if (p->tile[2] <= 0) sm = std::max(sm, zt.smem);
+                    kernel<<<g, 2 * TX * G, sm, st>>>(in, out, d, twz, spec, sc, TX);
+                };
                 if (back && sc.msa) {
                     ensure_smem<k_zback_p<T, N1, N2, true>>();
-                    k_zback_p<T, N1, N2, true><<<g, 2 * TX * G, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);
+                    go(k_zback_p<T, N1, N2, true>, B10, Bs);
                 } else if (back) {
                     ensure_smem<k_zback_p<T, N1, N2>>();
-                    k_zback_p<T, N1, N2><<<g, 2 * TX * G, sm, st>>>(B10, Bs, d, twz, spec, sc, TX);
+                    go(k_zback_p<T, N1, N2>, B10, Bs);
                 } else {
                     ensure_smem<k_zmac_p<T, N1, N2>>();
-                    k_zmac_p<T, N1, N2><<<g, 2 * TX * G, sm, st>>>(Bs, B10, d, twz, spec, sc, TX);
+                    go(k_zmac_p<T, N1, N2>, Bs, B10);
                 }
             })) {
             dim3 gz((d.Wx + l.TX_z - 1) / l.TX_z, d.Ly);

@@ -75,6 +75,13 @@ struct MuEnds {
     int args[2] = {0, 0};
 };
 
+// columns per CTA of a z kernel by the built-in rule and the shared memory it
+// asks for at least (0 columns: not asked yet)
+struct ZRule {
+    int tx = 0;
+    size_t smem = 0;
+};
+
 struct Problem {
     // ---- descriptor (copied) ----
     int nx = 0, ny = 0, nz = 0;
@@ -132,6 +139,7 @@ struct Problem {
     MuEnds *ends = nullptr;           // set while one is recorded
     int mg_levels = 0;
     int tile[3] = {0, 0, 0};          // register-FFT CTA tiles (x lines, y columns, z columns); 0: rule
+    ZRule ztile[3][2];                // by PNP_PREC_FP64, FP32, DF64 and direction
     double tuned_ms = 0;              // mu_ex time measured by the autotuner
 
     size_t npts() const { return (size_t)nx * ny * nz; }

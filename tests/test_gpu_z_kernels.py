@@ -62,3 +62,20 @@ def test_small_planes_in_fp32_match_oracle(pnp, length):
                                           ((90, 90), 40), ((64, 64), 64), ((64, 64), 40), ((32, 64), 128)])
 def test_column_tiles_match_oracle(pnp, plane, length):
     check(pnp, plane, length, 3, ("fp64", "df64", "fp32"))
+
+
+@pytest.mark.parametrize("length", [64, 96, 128])
+def test_msa_column_tiles_match_oracle(pnp, length):
+    """The z back with the MSA term keeps the paired-column form and a tile of its own."""
+    spec, _ = mu_microbench(shape=(6, 7, length - 8))
+    spec.msa, spec.fft_len = True, (40, 48, length)
+    rng = np.random.default_rng(length)
+    rho = np.stack([r * rng.lognormal(0.0, 0.1, spec.shape) for r in BULK[:3]])
+    ref, bad = oracle.excess_mu(spec, rho)
+    assert bad == 0
+    with pnp.Problem(spec) as P:
+        for precision in ("fp64", "df64", "fp32"):
+            for _ in range(2):
+                mu = P.excess_mu(rho, precision=precision)
+                for i in range(3):
+                    assert np.abs(mu[i] - ref[i]).max() <= TOL[precision] * np.abs(ref[i]).max(), precision
