@@ -125,8 +125,10 @@ enum { PNP_PREC_DEFAULT = -1, PNP_PREC_FP64 = 0, PNP_PREC_FP32 = 1, PNP_PREC_DF6
  * marks the boundaries of the phases of every Gummel iteration with the GPU's
  * nanosecond global timer (one single-thread kernel per boundary) and sums
  * the time spent in each phase; pnp_gummel_phase_times reads the sums of the
- * last solve.  Results are unchanged; the marks add a few microseconds per
- * iteration. */
+ * last solve.  So that the phases have boundaries, mu_ex runs before the Poisson
+ * step in these solves, not beside it as in others: an iteration takes longer by
+ * up to the shorter of the two, and the phases add up to the time of the marked
+ * iteration, not of an unmarked one.  Results are unchanged. */
 #define PNP_FLAG_PHASE_TIMING 16u
 
 /* hard-sphere functional (Sec 2.3.1): Rosenfeld's, whose derivatives the
@@ -326,8 +328,8 @@ int pnp_gummel_solve(pnp_problem *p, const double *phi0, const double *rho0, dou
 /* Per-phase device time of the last pnp_gummel_solve of a problem created
  * with PNP_FLAG_PHASE_TIMING, summed over its Gummel iterations: ms[0] mu_ex,
  * ms[1] the Poisson step (right-hand side, multigrid-preconditioned CG, phi
- * relaxation), ms[2] the Nernst-Planck solves and density updates of every
- * species, ms[3] the end of the iteration (Anderson mixing when enabled, the
+ * relaxation), ms[2] the Nernst-Planck solves (side by side) and density updates of
+ * every species, ms[3] the end of the iteration (Anderson mixing when enabled, the
  * residual and the loop decision).  Fills min(max_phases, 4) entries and
  * returns 4; the equilibrium stage is not included.  Synchronises.  Errors:
  * PNP_ERR_INVALID (no flag, no solve yet, bad arguments), PNP_ERR_CUDA. */
