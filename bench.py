@@ -268,8 +268,10 @@ def stage_flops(name, dims, s):
 # the 128^3 workload by the rows it moves; set to None whenever the kernel
 # changes after the capture.
 PROFILED_TRAFFIC = {
-    ("fp64", "z_back"): 1.1299e9,     # k_zback_p_fp64_120_pad256.md
-    ("fp32", "z_back"): None,
+    # k_zback_p_fp64_120_pad256.md: 1074.8 MB at 120^3 x 1136.8 / 1081.8 (algorithmic)
+    ("fp64", "z_back"): 1.1294e9,
+    # k_zreg_fp32_120_pad256.md: 528.9 MB at 120^3 x 568.4 / 540.9
+    ("fp32", "z_back"): 5.557e8,
     # k_zq4_dd_120_pad256.md: 1054.9 / 1083.1 MB at 120^3, x (algorithmic
     # bytes at 128^3 / at 120^3) = 1137 / 1082 MB
     ("df64", "z_mac"): 1.1085e9,

@@ -444,7 +444,7 @@ int pnp_weight_stencil(int kind, double r_in, double r_out, int nmu, int ntheta,
  * and h_nm), by the ball quadrature of Sec 3.5 with the descriptor's counts,
  * each node deposited trilinearly.  out gets (2S+1)^3 values in the layout
  * of pnp_weight_stencil; S >= ceil(s) + 1.  The set-up stencil of the
- * electrostatic-correlation term; the device pipeline does not apply it yet.
+ * electrostatic-correlation term that PNP_FLAG_MSA adds to mu_ex.
  * Errors: PNP_ERR_INVALID. */
 int pnp_msa_stencil(const pnp_problem_desc *desc, int i, int j, int S, double *out);
 

@@ -315,8 +315,10 @@ __global__ void k_diag(Op A, double *__restrict__ dgn, double *__restrict__ idg)
 //
 // 11 FP64 operations a point instead of 24 on half-idle warps: a 96^3 colour is
 // FP64-bound, and 128-thread CTAs put the 512 warps of a 32^3 colour on 128 SMs,
-// one warp on each quarter of an SM.  With the rest of this file a CG iteration
-// went from 343 to 103 us at 32^3 and from 700 to 290 us at 96^3.
+// one warp on each quarter of an SM.  A 96^3 colour takes 10.7 us with its
+// operands in L2 (its operations alone: 9.2 at the measured FP64 rate) and 14.7 from
+// HBM.  With the rest of this file a CG iteration went from 343 to 103 us at 32^3
+// and from 700 to 290 us at 96^3.
 //
 // RES: the residual of the swept points is written too.  Their neighbours do not
 // change before the restriction, so the sum just formed serves it: three more
@@ -623,7 +625,8 @@ __global__ void k_pcg_check(LinCtl *ctl, const double *__restrict__ part_rr, int
 // __syncthreads: iterate, right-hand side, residual, coefficients and neighbour
 // places of every level stay in shared memory, split by colour, so a warp reads
 // and writes consecutive words.  512 points of one colour are 16 warps, four on
-// each quarter of the SM: 4 x 11 FP64 instructions of 76 clocks, 1.6 us a phase;
+// each quarter of the SM: 4 x 11 FP64 instructions of 64 clocks, 1.4 of the 1.6 us
+// that a phase takes;
 // a 12^3 level (2.8 us) is faster as chip-wide launches, so the line is 1024
 // points.  The coarsest level (at most kCoarseWarp points) runs its 40
 // symmetric sweeps in one warp, in registers.

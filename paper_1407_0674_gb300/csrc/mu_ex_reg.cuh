@@ -355,9 +355,10 @@ __device__ __forceinline__ void load_spec(T (&g)[kChunk][N1], const T *__restric
     }
 }
 
-// Zero-extended columns of at most half the length skip the zero butterflies in
-// the 64-bit paired-column kernels; in FP32 the second form of the stage costs
-// more than it saves (z MAC of 48 points on 64 x 64 columns 33 -> 39 us).
+// Zero-extended columns of at most half the length skip the zero butterflies of
+// the radix-16 stage of 256 points, the only one that has a half form, in the 64-bit
+// paired-column kernels.  FP32 columns of that length take the kernels with
+// register state below, with up to three species.
 template <typename T, int L> __device__ __forceinline__ bool half_column(int nz) {
     return !std::is_same<T, float>::value && 2 * nz <= L;
 }
@@ -797,10 +798,10 @@ namespace pnp {
 // its S x N1 accumulators (z back) or transformed density values (z MAC) in
 // registers instead of a shared-memory slot per product, the lane twiddles
 // come from a shared table, and each kernel type's spectra for the CTA's
-// columns are staged in shared memory by cp.async while the first column of
-// the type is transformed.  Problems with the MSA term keep k_zback_p (its
-// extra pair loop would spill here).  Measured at 128^3 -> 256^3: z back 0.648 -> 0.549
-// ms, z MAC 0.505 -> 0.487 ms against k_zback_p / k_zmac_p.
+// columns are staged in shared memory by cp.async, in two buffers, while the
+// type before is worked on.  Problems with the MSA term keep k_zback_p (its
+// extra pair loop would spill here).  Measured at 128^3 -> 256^3: z back 0.500 ms, z MAC
+// 0.460, against 0.648 and 0.505 for k_zback_p / k_zmac_p.
 
 __device__ __forceinline__ void cp_async_f32(float *smem, const float *gmem, bool valid) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
