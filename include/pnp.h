@@ -252,7 +252,7 @@ int pnp_plan_problem(const pnp_problem_desc *desc, pnp_problem_info *info, doubl
  * term (Sec 2.3.2).  Writes mu_ex [s][nz][ny][nx] (host).  Blocks until done.
  * The densities are checked on the device: negative or non-finite ones are
  * refused (PNP_ERR_INVALID) with mu_ex and a status pending from earlier device
- * calls left as they were, but a call of fewer than 2^22 values may have taken
+ * calls left as they were, but a call of fewer than 2^24 values may have taken
  * the time of a full one by then.
  * Errors: PNP_ERR_INVALID, PNP_ERR_PACKING (n3 >= 1 somewhere), PNP_ERR_NOMEM,
  * PNP_ERR_CUDA. */

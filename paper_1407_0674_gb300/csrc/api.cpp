@@ -378,11 +378,11 @@ int pnp_excess_mu(pnp_problem *h, const double *rho, double *mu_ex, int precisio
     // of the copy back were 0.55 and 0.40 of the 0.86 ms of a 64^3 FP32 call.
     // Nothing is copied back for densities that fail the check.  mu_ex starts
     // without waiting for the verdict (waiting: 64^3 343 -> 364 us, 32^3 95 ->
-    // 111), except where a refusal would have spent much more on it than the wait
-    // (kCheckFirst values: calls of 1.2 ms and more), or where a device call on
+    // 111), except where a valid call does not notice the wait and a refused one
+    // would have run for long (kCheckFirst values: 4 ms and more), or where a device call on
     // another stream may be at work in the workspace, which only a call that is
     // taken may disturb.
-    constexpr size_t kCheckFirst = (size_t)1 << 22;
+    constexpr size_t kCheckFirst = (size_t)1 << 24;
     cudaStream_t st = p->stream;
     cudaError_t e = cudaMemcpyAsync(p->d_io, rho, sizeof(double) * n, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return fail(cuda_status(e));

@@ -174,10 +174,11 @@ def test_graph_calls_of_every_option(pnp, case, precision):
             assert torch.equal(out, want), k
 
 
-@pytest.mark.parametrize("shape", [(10, 10, 10), (112, 112, 112)])    # before and after the check's verdict
+@pytest.mark.parametrize("shape", [(10, 10, 10), (112, 112, 112)])
 def test_refused_host_call_changes_nothing(pnp, shape):
     """Refused densities leave a pending device status, the output and the next result as
-    they were, and are refused for what they are when memory runs out too."""
+    they were, and are refused for what they are when memory runs out too.  After a call
+    on another stream the verdict is waited for before anything else runs."""
     import torch
     spec, rho = mu_microbench(shape=shape)
     bad = rho.copy()
